@@ -37,7 +37,7 @@
 //               after building chunk i they run the chain of chunk i - 2
 //               (thread j = candidate j = TMEM lane j of the D2 buffer), so
 //               that the epilogue only forms E;
-//   warp 12     MMA issuer (lane 0): MMA 1 of unit u + 1, then MMA 2 of unit u
+//   warp 12     MMA issuer (one lane): MMA 1 of unit u + 1, then MMA 2 of unit u
 //               (TMEM: S / E buffers u & 1 at columns 128 (u & 1); D2 buffers
 //               i & 1 at 256 + NPSI (i & 1), accumulated over the chunk's units);
 //   warps 4-11  epilogue: warp w owns lanes 32 (w % 4) .. + 31 and columns
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
     if (!ok && lane == 0) fail();
   } else if (warp == 12) {
     // ---- MMA issuer
-    if (lane == 0 && U > 0) {
+    if (elect_one() && U > 0) {
       constexpr uint32_t IDESC1 = idesc_f16(S::UQ);
       constexpr uint32_t IDESC2 = idesc_f16(NPSI);
       // descriptor bases (a descriptor for base + off is base + off / 16)

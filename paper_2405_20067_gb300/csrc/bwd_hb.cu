@@ -37,7 +37,7 @@
 //   warps 0-3   builders: coefficient rows of chunk i into coefficient stage
 //               i % CS, the chunk's per-candidate data (m~, w / rho, entry,
 //               row factor, rho) into stash slot i % SS;
-//   warp 12     MMA issuer (lane 0): MMA 1 of unit u + LEAD, then MMA 2 of u;
+//   warp 12     MMA issuer (one lane): MMA 1 of unit u + LEAD, then MMA 2 of u;
 //   warps 4-11  epilogue: warp w owns TMEM lanes 32 (w % 4) .. + 31 (its
 //               candidates) and 64 columns (queries) of each unit; after the
 //               last unit of chunk i it forms half of the record parts of
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
     if (!ok && lane == 0) fail();
   } else if (warp == 12) {
     // ---- MMA issuer
-    if (lane == 0 && U > 0) {
+    if (elect_one() && U > 0) {
       constexpr uint32_t IDESC1 = idesc_f16(S::UQ);
       // MMA 2: B = Phi read MN-major (features on N); instruction bit 16
       constexpr uint32_t IDESC2 = idesc_f16(ND) | (1u << 16);
