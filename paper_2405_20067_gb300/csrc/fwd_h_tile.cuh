@@ -17,25 +17,32 @@
 //     stage carries a flag so that chunks without such rows skip it).
 //
 // CTA = one tile of up to 256 queries (two M = 128 row blocks sharing the
-// candidate operand), 416 threads, one CTA per SM (it owns all 512 TMEM
-// columns: two accumulator buffers x two row blocks x 128 candidates):
-//   warps 0-3   builders: thread j turns candidate j of a chunk of 128 into
-//               its coefficient row (FP16 hi / lo, K-major no-swizzle layout)
-//               and weight pair entry in one of CS shared-memory stages; the
-//               records of the next chunk are loaded into registers meanwhile;
-//               each warp then arrives on coef_full;
-//   warp 12     MMA issuer: lane 0 issues the MMAs of chunk i once its stage
-//               is full and accumulator buffer i & 1 is free, and commits
-//               them to acc_full and coef_empty (a warp of its own, so that
-//               issuing overlaps the building of the next chunks);
-//   warps 4-11  epilogue: warps 4-7 serve row block 0, warps 8-11 row block 1
-//               (each block has its own accumulator barriers, so the two
-//               groups run independently); warp w reads TMEM lanes 32 (w % 4)
-//               .. + 31 of its block at all 128 columns with the 16x256b load
-//               shape (a thread holds 4 rows x 2 columns of every 8-column
-//               group), the loads of the next 32 columns in flight while the
-//               current ones are used; it forms e = 2^s and accumulates w e;
-//               row sums are completed with shuffles at the end.
+// candidate operand), 416 threads, one CTA per SM.  What bounds the tile is
+// the shared-memory pipe, which the MMAs' operand reads (one wavefront per
+// 128 bytes), the weight loads and the coefficient rows share; it was 68%
+// (N = 6) to 82% (N = 10) busy, and every barrier or load behind it waited
+// ~400 cycles, while Phi was an operand in shared memory and each weight
+// load served four query rows.  So Phi, the same for all of a tile's chunks,
+// is the A operand in tensor memory (hi and lo; N >= 10 has room for hi only
+// and keeps lo in shared memory), the chunks are of 96 candidates so that two
+// double-buffered accumulators and Phi share the 512 columns (an MMA of 96
+// columns costs its share of one of 128), and a weight load serves eight rows.
+// Measured: N = 10 480 x 272 frame (100,000 Gaussians) 6.78 -> 6.00 ms, N = 10
+// fit 14.6 -> 12.6 ms, N = 8 5,000 Gaussians 159 -> 136 us.
+//   warps 0-3   builders: a warp turns its 32 candidates of a chunk into
+//               coefficient rows (FP16 hi / lo, K-major no-swizzle layout)
+//               and weight pair entries in one of CS shared-memory stages
+//               and arrives on coef_full;
+//   warp 12     MMA issuer: one lane issues the MMAs of chunk i once its
+//               stage is full and accumulator buffer i & 1 is free, and
+//               commits them to acc_full and coef_empty (a warp of its own,
+//               so that issuing overlaps the building of the next chunks);
+//   warps 4-11  epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 of both
+//               row blocks at half of the chunk's columns with the 16x256b
+//               load shape (a thread holds 4 rows x 2 columns of every
+//               8-column group); it forms e = 2^s and accumulates w e; row
+//               sums are completed with shuffles and, over the two column
+//               halves, through shared memory at the end.
 // Barrier operations are one per warp (an elected lane), and every wait is
 // bounded: on a timeout the kernel records NDG_ERR_TIMEOUT, lets the issued
 // MMAs finish (bounded), frees its tensor memory and returns.
@@ -55,27 +62,32 @@ struct FwdHShape {
   static constexpr int P = tri(N);
   static constexpr int F = P + N + 1;
   static constexpr int KP = (F + 15) / 16 * 16;  // K step of kind::f16 is 16
-  static constexpr int NC = 128;                 // candidates per chunk (MMA N)
+  static constexpr int NC = 96;                  // candidates per chunk (MMA N)
+  static constexpr int GPC = NC / 32;            // builder groups (one warp's 32) per chunk
   static constexpr int R = rec_floats(N);
   static constexpr uint32_t SBO = (KP / 8) * 128;  // 8-row group stride (bytes)
-  static constexpr uint32_t PHI_BYTES = 256u * KP * 2;  // one of hi / lo, 256 rows
-  static constexpr uint32_t HALF_BYTES = 128u * KP * 2; // one 128-row block
+  // tensor memory: four accumulators (buffer, row block) of NC columns, then
+  // Phi as the MMAs' A operand, KP / 2 columns per row block and half: hi of
+  // both blocks, and lo too where the 512 columns hold it (N <= 9)
+  static constexpr uint32_t TM_PHI = 4u * NC;
+  static constexpr bool LO_TM = TM_PHI + 2 * KP <= 512;
+  static_assert(TM_PHI + KP <= 512, "tensor memory");
+  static constexpr uint32_t PHI_BYTES = LO_TM ? 0 : 256u * KP * 2;  // lo half in shared memory
+  static constexpr uint32_t HALF_BYTES = 128u * KP * 2;  // one 128-row block of it
   static constexpr uint32_t B_BYTES = (uint32_t)NC * KP * 2;
   static constexpr uint32_t W_BYTES = (uint32_t)NC * 16;  // w0 w0' w1 w1' w2 w2' k k' per pair
   static constexpr uint32_t C_STAGE = 2 * B_BYTES + W_BYTES;
   // coefficient stages: as many as fit next to Phi (at most 4; 2 KB are left
   // for the static shared variables).  The builders run up to CS chunks ahead
-  // of the epilogue, which frees a stage only at the end of its chunk, so
-  // two stages leave the builders idle for a whole chunk (measured at N = 10:
-  // a third stage is worth about a fifth of the time).
-  static constexpr uint32_t STAGE_ROOM = 227u * 1024u - 2048u - 2 * PHI_BYTES - 128u;
+  // of the epilogue, which frees a stage only at the end of its chunk.
+  static constexpr uint32_t STAGE_ROOM = 227u * 1024u - 2048u - PHI_BYTES - 128u;
   static constexpr int CS = STAGE_ROOM / C_STAGE >= 4 ? 4 : (int)(STAGE_ROOM / C_STAGE);
-  static constexpr uint32_t SMEM_USED = 2 * PHI_BYTES + CS * C_STAGE + 128;
+  static constexpr uint32_t SMEM_USED = PHI_BYTES + CS * C_STAGE + 128;
   // more than half of the SM's shared memory: one CTA per SM
   static constexpr uint32_t SMEM = SMEM_USED > 116u * 1024u ? SMEM_USED : 116u * 1024u;
   static_assert(SMEM <= 227u * 1024u, "shared memory");
   static_assert(CS >= 2, "coefficient stages");
-  static_assert(NC == 128, "candidate mapping");
+  static_assert(2 * B_BYTES >= 256 * 12, "row sums of the second column half");
 };
 
 namespace {
@@ -95,23 +107,6 @@ __device__ __forceinline__ uint32_t kmajor_off_h(int row, int k, uint32_t sbo) {
          (uint32_t)(k & 7) * 2u;
 }
 
-// Writes one K-major row of KP values (multiple of 8) as FP16 hi / lo.
-template <int KP>
-__device__ __forceinline__ void store_row_h(uint8_t* hi, uint8_t* lo, int row, uint32_t sbo,
-                                            const float (&v)[KP]) {
-#pragma unroll
-  for (int k = 0; k < KP; k += 8) {
-    uint4 h, l;
-    split_h2(v[k], v[k + 1], h.x, l.x);
-    split_h2(v[k + 2], v[k + 3], h.y, l.y);
-    split_h2(v[k + 4], v[k + 5], h.z, l.z);
-    split_h2(v[k + 6], v[k + 7], h.w, l.w);
-    const uint32_t off = kmajor_off_h(row, k, sbo);
-    *reinterpret_cast<uint4*>(hi + off) = h;
-    *reinterpret_cast<uint4*>(lo + off) = l;
-  }
-}
-
 constexpr float kNegHalfLog2eH = -0.72134752044448170368f;
 constexpr float kRowMax = 16384.0f;  // coefficient rows are kept below 2^14 (FP16 max 65504)
 
@@ -120,12 +115,11 @@ constexpr float kRowMax = 16384.0f;  // coefficient rows are kept below 2^14 (FP
 // Barriers and small shared state of one tile, sized for the largest shape
 // (CS <= 4 coefficient stages, N <= 12).
 struct FwdHSync {
-  // accumulator barriers per (buffer, row block): index 2 b + h
-  uint64_t coef_full[4], coef_empty[4], acc_full[4], acc_empty[4], drain;
+  uint64_t coef_full[4], coef_empty[4], acc_full[2], acc_empty[2], drain;
   uint32_t tmem_base;
   float sred[8 * 12 * 2];
   float sctr[12], sh[12];
-  __align__(16) int sflag[4][4];
+  __align__(16) int sflag[4][4];  // per stage and 32-candidate group: a row was scaled
   int s_abort;
 };
 
@@ -139,8 +133,7 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
   using S = FwdHShape<N>;
   constexpr int P = S::P, KP = S::KP, NC = S::NC, CS = S::CS, R = S::R, R4 = R / 4;
   static_assert(CS <= 4 && N <= 12, "FwdHSync sizes");
-  uint8_t* Ahi = base;
-  uint8_t* Alo = Ahi + S::PHI_BYTES;
+  uint8_t* Alo = base;                // Phi lo, where tensor memory does not hold it
   uint8_t* Cst = Alo + S::PHI_BYTES;  // CS stages of (Bhi, Blo, weights)
   uint64_t* coef_full = sy.coef_full;
   uint64_t* coef_empty = sy.coef_empty;
@@ -161,12 +154,12 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
   // ---- setup: barriers, tile centre and scales, Phi rows (epilogue warps)
   if (tid == 0) {
     for (int i = 0; i < CS; ++i) {
-      mbar_init(&coef_full[i], 4);
-      mbar_init(&coef_empty[i], 1 + 4 * nh);  // issuer commit + the busy epilogue warps
+      mbar_init(&coef_full[i], S::GPC);
+      mbar_init(&coef_empty[i], 1 + 8);  // issuer commit + the epilogue warps
     }
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 2; ++i) {
       mbar_init(&acc_full[i], 1);
-      mbar_init(&acc_empty[i], 4);
+      mbar_init(&acc_empty[i], 8);
     }
     mbar_init(&drain, 1);
     s_abort = 0;
@@ -219,7 +212,22 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
     phi[P + N] = active_row ? 1.0f : 0.0f;
 #pragma unroll
     for (int k = P + N + 1; k < KP; ++k) phi[k] = 0.0f;
-    store_row_h<KP>(Ahi, Alo, row, S::SBO, phi);
+    // row `row` = lane 32 (warp % 4) + lane of row block (warp - 4) / 4
+    const uint32_t ph = sy.tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + S::TM_PHI +
+                        (uint32_t)(((warp - 4) >> 2) * (KP / 2));
+    fence_after_sync();
+#pragma unroll
+    for (int k = 0; k < KP; k += 8) {
+      uint4 h, l;
+      split_h2(phi[k], phi[k + 1], h.x, l.x);
+      split_h2(phi[k + 2], phi[k + 3], h.y, l.y);
+      split_h2(phi[k + 4], phi[k + 5], h.z, l.z);
+      split_h2(phi[k + 6], phi[k + 7], h.w, l.w);
+      tmem_st4(ph + (uint32_t)(k / 2), h);
+      if constexpr (S::LO_TM) tmem_st4(ph + (uint32_t)(KP + k / 2), l);
+      else *reinterpret_cast<uint4*>(Alo + kmajor_off_h(row, k, S::SBO)) = l;
+    }
+    tmem_wait_st();
   }
   fence_proxy_async();
   fence_before_sync();
@@ -234,15 +242,22 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
     if (a.status) set_status(a.status, NDG_ERR_TIMEOUT);
   };
 
+  // epilogue warps 4-7: the thread's query row inside each row block, and its
+  // rows' sums
+  const int my_row = (warp & 3) * 32 + ((lane & 3) >> 1) * 16 + (lane & 1) * 8 + (lane >> 2);
+  float rs[2][3] = {};
+
   if (warp < 4) {
     // ---- builders
-    const int j = tid;
+    // warp w builds the 32-candidate groups w, w + 4, ...; group g is rows
+    // 32 (g % GPC) .. + 31 of chunk g / GPC
+    const int ngroups = nchunks * S::GPC;
     float hsc[N];
 #pragma unroll
     for (int d = 0; d < N; ++d) hsc[d] = sh[d];
-    auto cand = [&](int i) -> int {
-      const long long c = beg + (long long)i * NC + j;
-      const int g = (i < nchunks && c < end) ? a.ids[c] : -1;
+    auto cand = [&](int gr) -> int {
+      const long long c = beg + (long long)gr * 32 + lane;
+      const int g = c < end ? a.ids[c] : -1;
       return ((unsigned)g < (unsigned)a.Ge) ? g : -1;
     };
     const int stride4 = a.rec_stride4 > 0 ? a.rec_stride4 : R4;
@@ -256,18 +271,19 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
         for (int k = 0; k < R4; ++k) r[k] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
     };
-    // N <= 6: the records of chunk i + 1 are loaded into registers while
-    // chunk i is built; larger records are loaded right after a build (the
+    // N <= 6: the records of the warp's next group are loaded into registers
+    // while a group is built; larger records are loaded right after a build (the
     // latency overlaps the next stage wait) to keep the register count down.
     constexpr bool PRE = N <= 6;
     float4 cur[R4], nxt[PRE ? R4 : 1];
-    load(cand(0), cur);
-    int g_next = cand(1);
-    for (int i = 0; i < nchunks; ++i) {
-      const int s = i % CS;
+    load(cand(warp), cur);
+    int g_next = cand(warp + 4);
+    for (int gr = warp; gr < ngroups; gr += 4) {
+      const int i = gr / S::GPC, s = i % CS;
+      const int j = (gr - i * S::GPC) * 32 + lane;
       if constexpr (PRE) {
-        load(g_next, nxt);  // chunk i + 1 (zeros past the end)
-        g_next = cand(i + 2);
+        load(g_next, nxt);  // the warp's next group (zeros past the end)
+        g_next = cand(gr + 8);
       }
       bool ok = true;
       if (i >= CS) ok = warp_wait(&coef_empty[s], ((i / CS) - 1) & 1, abort_flag);
@@ -347,180 +363,195 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
         wd[6] = back;
       }
       const bool any_scaled = __any_sync(0xffffffffu, scaled);
-      if (lane == 0) sflag[s][warp] = any_scaled ? 1 : 0;
+      if (lane == 0) sflag[s][gr - i * S::GPC] = any_scaled ? 1 : 0;
       fence_proxy_async();
       warp_arrive(&coef_full[s]);
       if constexpr (PRE) {
 #pragma unroll
         for (int k = 0; k < R4; ++k) cur[k] = nxt[k];
       }
-      // one decision per warp
-      if (__shfl_sync(0xffffffffu, (!ok || *abort_flag) ? 1 : 0, 0)) break;
+      // a CTA that gives up stops every role at its next blocked wait
+      if (!ok) break;
       if constexpr (!PRE) {
-        load(g_next, cur);  // chunk i + 1
-        g_next = cand(i + 2);
+        load(g_next, cur);  // the warp's next group
+        g_next = cand(gr + 8);
       }
     }
   } else if (warp == 12) {
     // ---- MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       // descriptor bases (a descriptor for base + off is base + off / 16)
-      const uint64_t dA0 = smem_desc(smem_u32(Ahi), 128, S::SBO);
+      const uint64_t dA0 = smem_desc(smem_u32(Alo), 128, S::SBO);
       const uint64_t dB0 = smem_desc(smem_u32(Cst), 128, S::SBO);
-      constexpr uint64_t A_LO = S::PHI_BYTES >> 4, B_LO = S::B_BYTES >> 4;
+      constexpr uint64_t B_LO = S::B_BYTES >> 4;
       constexpr uint32_t IDESC = idesc_f16(NC);
       for (int i = 0; i < nchunks; ++i) {
         const int s = i % CS, b = i & 1;
         bool ok = mbar_wait_sleep(&coef_full[s], (i / CS) & 1, abort_flag);
-        const uint64_t dbh = dB0 + (uint64_t)((s * S::C_STAGE) >> 4);
-        for (int h = 0; ok && h < nh; ++h) {
-          // row block h of buffer b is free once its epilogue group has read chunk i - 2
-          if (i >= 2) ok = mbar_wait_sleep(&acc_empty[2 * b + h], ((i >> 1) - 1) & 1, abort_flag);
-          if (!ok) break;
-          fence_after_sync();
-          const uint32_t d = tmem + (uint32_t)(b * 256 + h * 128);
-          const uint64_t dah = dA0 + (uint64_t)((h * S::HALF_BYTES) >> 4);
-#pragma unroll
-          for (int ks = 0; ks < KP / 16; ++ks) {
-            const uint64_t ko = (uint64_t)ks * 16u;  // two 16-byte core matrices per K step
-            mma_f16(d, dah + ko, dbh + ko, IDESC, ks > 0 ? 1u : 0u);
-            mma_f16(d, dah + ko, dbh + B_LO + ko, IDESC, 1u);
-            mma_f16(d, dah + A_LO + ko, dbh + ko, IDESC, 1u);
-          }
-          mma_commit(&acc_full[2 * b + h]);
-        }
+        // buffer b is free once the epilogue has read chunk i - 2
+        if (ok && i >= 2) ok = mbar_wait_sleep(&acc_empty[b], ((i >> 1) - 1) & 1, abort_flag);
         if (!ok) {
           fail();
           break;
         }
+        fence_after_sync();
+        const uint64_t dbh = dB0 + (uint64_t)((s * S::C_STAGE) >> 4);
+        for (int h = 0; h < nh; ++h) {
+          const uint32_t d = tmem + (uint32_t)((2 * b + h) * NC);
+          const uint32_t ah = tmem + S::TM_PHI + (uint32_t)(h * (KP / 2));
+          const uint64_t dal = dA0 + (uint64_t)((h * S::HALF_BYTES) >> 4);
+#pragma unroll
+          for (int ks = 0; ks < KP / 16; ++ks) {
+            const uint64_t ko = (uint64_t)ks * 16u;  // two 16-byte core matrices per K step
+            mma_f16_ts(d, ah + 8u * ks, dbh + ko, IDESC, ks > 0 ? 1u : 0u);
+            mma_f16_ts(d, ah + 8u * ks, dbh + B_LO + ko, IDESC, 1u);
+            if constexpr (S::LO_TM) mma_f16_ts(d, ah + KP + 8u * ks, dbh + ko, IDESC, 1u);
+            else mma_f16(d, dal + ko, dbh + ko, IDESC, 1u);
+          }
+        }
+        mma_commit(&acc_full[b]);
         mma_commit(&coef_empty[s]);
       }
     }
   } else {
     // ---- epilogue (tcgen05.ld 16x256b: thread t holds lanes t/4 and t/4 + 8
-    // of a 16-lane half at columns 2 (t % 4) + {0, 1} of every 8-column group,
-    // so each weight load serves four query rows)
-    const int quad = warp & 3, h = (warp - 4) >> 2;
-    const int tq = lane & 3, tr = lane >> 2;
-    // rows ri = hb * 2 + r8: 16-lane half hb, lane t/4 + 8 r8; .x / .y
-    // accumulate the even / odd column of the thread's pairs
-    float2 acc[4][3];
+    // of a 16-lane half at columns 2 (t % 4) + {0, 1} of every 8-column group).
+    // The warp takes its 32 lanes of both row blocks, so that one load of a
+    // pair of weights serves eight query rows.
+    constexpr int CW = NC / 2, NB = CW / 16;  // this warp's columns, in blocks of 16
+    const int quad = warp & 3, ch = (warp - 4) >> 2;
+    const int tq = lane & 3;
+    // rows ri = 4 h + 2 hb + r8: row block h, 16-lane half hb, lane t/4 + 8 r8;
+    // .x / .y accumulate the even / odd column of the thread's pairs
+    float2 acc[8][3];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 8; ++r)
 #pragma unroll
       for (int c = 0; c < 3; ++c) acc[r][c] = make_float2(0.f, 0.f);
-    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(h * 128);
-    // 32-column block n of buffer b: both 16-lane halves
-    auto load = [&](int b, int n, uint32_t (&v)[2][16]) {
-#pragma unroll
-      for (int hb = 0; hb < 2; ++hb)
-        tmem_ld16x256_x4_nowait(lane_base + ((uint32_t)(hb * 16) << 16) + (uint32_t)(b * 256 + n * 32),
-                                v[hb]);
-    };
-    // accumulate block n (columns 32 n + 8 k + 2 tq + {0, 1}, k = 0..3): the
-    // 32 exponentials first, in place (independent MUFU operations whose
-    // latency overlaps), then the colour sums
-    auto use = [&](const float* wp, int n, uint32_t (&v)[2][16], auto sc_tag) {
+    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ch * CW);
+    // one chunk: units (block n, row block h) in the order n-major, the next
+    // unit loading while one is used
+    auto chunk = [&](int b, const float* wp, auto sc_tag, auto nh_tag) {
       constexpr bool SC = decltype(sc_tag)::value;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        float2 sc = make_float2(1.f, 1.f);
-        if (SC) sc = *reinterpret_cast<const float2*>(wp + (16 * n + 4 * k) * 8 + 6);
-#pragma unroll
-        for (int hb = 0; hb < 2; ++hb)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            float sv = __uint_as_float(v[hb][4 * k + j]);
-            if (SC) sv *= (j & 1) ? sc.y : sc.x;
-            v[hb][4 * k + j] = __float_as_uint(ex2_approx(sv));
-          }
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float* wk = wp + (16 * n + 4 * k) * 8;
-        const float4 w01 = *reinterpret_cast<const float4*>(wk);
-        const float2 w2 = *reinterpret_cast<const float2*>(wk + 4);
+      constexpr int NH = decltype(nh_tag)::value, NU = NB * NH;
+      uint32_t v[2][2][8];
+      float4 w01[2];
+      float2 w2[2], sc[2];
+      auto load = [&](int u) {
 #pragma unroll
         for (int hb = 0; hb < 2; ++hb)
+          tmem_ld16x256_x2_nowait(lane_base + ((uint32_t)(hb * 16) << 16) +
+                                      (uint32_t)((2 * b + u % NH) * NC + (u / NH) * 16),
+                                  v[u & 1][hb]);
+      };
+      load(0);
 #pragma unroll
-          for (int r8 = 0; r8 < 2; ++r8) {
-            const float2 e = make_float2(__uint_as_float(v[hb][4 * k + 2 * r8]),
-                                         __uint_as_float(v[hb][4 * k + 2 * r8 + 1]));
-            const int ri = hb * 2 + r8;
-            acc[ri][0] = __ffma2_rn(make_float2(w01.x, w01.y), e, acc[ri][0]);
-            acc[ri][1] = __ffma2_rn(make_float2(w01.z, w01.w), e, acc[ri][1]);
-            acc[ri][2] = __ffma2_rn(w2, e, acc[ri][2]);
+      for (int u = 0; u < NU; ++u) {
+        const int n = u / NH, h = u % NH;
+        if (h == 0) {
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const float* wk = wp + (8 * n + 4 * k) * 8;
+            w01[k] = *reinterpret_cast<const float4*>(wk);
+            w2[k] = *reinterpret_cast<const float2*>(wk + 4);
+            if (SC) sc[k] = *reinterpret_cast<const float2*>(wk + 6);
           }
+        }
+        uint32_t(&vu)[2][8] = v[u & 1];
+        tmem_wait_ld();
+        tmem_reg_fence8(vu[0]);
+        tmem_reg_fence8(vu[1]);
+        if (u + 1 < NU) {
+          load(u + 1);
+        } else {
+          // this warp's reads of buffer b are complete
+          fence_before_sync();
+          warp_arrive(&acc_empty[b]);
+        }
+        // the unit's 16 exponentials first, in place (independent MUFU
+        // operations whose latency overlaps), then the colour sums
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int hb = 0; hb < 2; ++hb)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              float sv = __uint_as_float(vu[hb][4 * k + j]);
+              if (SC) sv *= (j & 1) ? sc[k].y : sc[k].x;
+              vu[hb][4 * k + j] = __float_as_uint(ex2_approx(sv));
+            }
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int hb = 0; hb < 2; ++hb)
+#pragma unroll
+            for (int r8 = 0; r8 < 2; ++r8) {
+              const float2 e = make_float2(__uint_as_float(vu[hb][4 * k + 2 * r8]),
+                                           __uint_as_float(vu[hb][4 * k + 2 * r8 + 1]));
+              const int ri = 4 * h + 2 * hb + r8;
+              acc[ri][0] = __ffma2_rn(make_float2(w01[k].x, w01[k].y), e, acc[ri][0]);
+              acc[ri][1] = __ffma2_rn(make_float2(w01[k].z, w01[k].w), e, acc[ri][1]);
+              acc[ri][2] = __ffma2_rn(w2[k], e, acc[ri][2]);
+            }
       }
     };
-    // one chunk: four 32-column blocks, block n + 1 loading while block n is used
-    auto chunk = [&](int b, const float* wp, auto sc_tag) {
-      uint32_t va[2][16], vb[2][16];
-      load(b, 0, va);
-      tmem_wait_ld();
-      tmem_reg_fence16(va[0]);
-      tmem_reg_fence16(va[1]);
-      load(b, 1, vb);
-      use(wp, 0, va, sc_tag);
-      tmem_wait_ld();
-      tmem_reg_fence16(vb[0]);
-      tmem_reg_fence16(vb[1]);
-      load(b, 2, va);
-      use(wp, 1, vb, sc_tag);
-      tmem_wait_ld();
-      tmem_reg_fence16(va[0]);
-      tmem_reg_fence16(va[1]);
-      load(b, 3, vb);
-      use(wp, 2, va, sc_tag);
-      tmem_wait_ld();
-      tmem_reg_fence16(vb[0]);
-      tmem_reg_fence16(vb[1]);
-      // this warp's reads of buffer b are complete
-      fence_before_sync();
-      warp_arrive(&acc_empty[2 * b + h]);
-      use(wp, 3, vb, sc_tag);
-    };
-    const bool my_block = h < nh;
-    for (int i = 0; my_block && i < nchunks; ++i) {
+    for (int i = 0; i < nchunks; ++i) {
       const int s = i % CS, b = i & 1;
-      bool ok = warp_wait(&acc_full[2 * b + h], (i >> 1) & 1, abort_flag);
-      if (ok) ok = warp_wait(&coef_full[s], (i / CS) & 1, abort_flag);
+      bool ok = warp_wait(&coef_full[s], (i / CS) & 1, abort_flag);
+      const int4 fl = *reinterpret_cast<const int4*>(&sflag[s][0]);
+      const bool scaled = (fl.x | fl.y | fl.z) != 0;
+      if (ok) ok = warp_wait(&acc_full[b], (i >> 1) & 1, abort_flag);
       if (!ok) {
         if (lane == 0) fail();
         break;
       }
       fence_after_sync();
-      const int4 fl = *reinterpret_cast<const int4*>(&sflag[s][0]);
-      const bool scaled = (fl.x | fl.y | fl.z | fl.w) != 0;
-      // weight pair entries of this thread: p = 16 n + 4 k + tq
-      const float* wp = reinterpret_cast<const float*>(Cst + s * S::C_STAGE + 2 * S::B_BYTES) + tq * 8;
-      if (scaled) chunk(b, wp, BoolTag<true>{});
-      else chunk(b, wp, BoolTag<false>{});
+      // weight pair entries of this thread: p = CW / 2 ch + 8 n + 4 k + tq
+      const float* wp = reinterpret_cast<const float*>(Cst + s * S::C_STAGE + 2 * S::B_BYTES) +
+                        (CW / 2 * ch + tq) * 8;
+      if (nh == 2) {
+        if (scaled) chunk(b, wp, BoolTag<true>{}, IntTag<2>{});
+        else chunk(b, wp, BoolTag<false>{}, IntTag<2>{});
+      } else {
+        if (scaled) chunk(b, wp, BoolTag<true>{}, IntTag<1>{});
+        else chunk(b, wp, BoolTag<false>{}, IntTag<1>{});
+      }
       warp_arrive(&coef_empty[s]);
     }
     // ---- row sums over the pair halves and the four threads sharing a lane
-    // (shuffles); thread tq writes row ri = tq
-    if (my_block && !*abort_flag) {
+    // (shuffles); thread tq keeps rows ri = tq and 4 + tq
 #pragma unroll
-      for (int ri = 0; ri < 4; ++ri) {
-        float rs[3];
+    for (int ri = 0; ri < 8; ++ri)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          float v = acc[ri][c].x + acc[ri][c].y;
-          v += __shfl_xor_sync(0xffffffffu, v, 1);
-          v += __shfl_xor_sync(0xffffffffu, v, 2);
-          rs[c] = v;
-        }
-        const int qr = h * 128 + quad * 32 + (ri >> 1) * 16 + (ri & 1) * 8 + tr;
-        if (ri == tq && qr < nq) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) a.y[(qt + qr) * 3 + c] = rs[c];
-        }
+      for (int c = 0; c < 3; ++c) {
+        float v = acc[ri][c].x + acc[ri][c].y;
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        if ((ri & 3) == tq) rs[ri >> 2][c] = v;
       }
+    // the second column half hands its sums over through the operand rows of
+    // stage 0 (every MMA that read them is complete: this warp saw the last
+    // chunk's acc_full, and no builder writes after it)
+    if (ch == 1 && !*abort_flag) {
+      float* dst = reinterpret_cast<float*>(Cst) + my_row * 3;
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dst[h * 128 * 3 + c] = rs[h][c];
     }
   }
   fence_before_sync();
   __syncthreads();
+  if (warp >= 4 && warp < 8 && !*abort_flag) {
+    const float* o = reinterpret_cast<const float*>(Cst) + my_row * 3;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (h * 128 + my_row < nq) {
+        const long long q = qt + h * 128 + my_row;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a.y[q * 3 + c] = nchunks > 0 ? rs[h][c] + o[h * 128 * 3 + c] : 0.0f;
+      }
+  }
   if (warp == 12 && lane == 0) {
     // every MMA this thread issued has completed once this commit arrives
     mma_commit(&drain);

@@ -80,6 +80,17 @@ __device__ __forceinline__ void tmem_ld16x256_x4_nowait(uint32_t taddr, uint32_t
       : "memory");
 }
 
+// 16x256b.x2 load without the wait: 16 lanes x 16 columns, as above with two
+// 8-column groups.
+__device__ __forceinline__ void tmem_ld16x256_x2_nowait(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+}
+
 // Empty register fence: values loaded by an asynchronous tcgen05.ld are
 // passed through here after tcgen05.wait::ld, so that no use of them can be
 // scheduled above the wait.
@@ -115,6 +126,12 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
       "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
+}
+// 32x32b.x4 store: thread t writes lane (base + t), 4 consecutive columns.
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint4& r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr),
+               "r"(r.x), "r"(r.y), "r"(r.z), "r"(r.w)
+               : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
