@@ -371,7 +371,7 @@ ndg_status ndg_forward_batch(const ndg_frame* frames, int n_frames, void* batch_
 
 /* Failure-detection self-test of the bounded device waits: launches one
  * CTA that waits on an mbarrier nothing ever completes, with the wait the
- * tensor-core kernels use (which = 0: the sleeping warp wait, about a
+ * tensor-core kernels use (which = 0: the roles' warp wait, about a
  * second; which = 1: the spinning wait of their final drain, about a second
  * or two).  When the bound runs out it records NDG_ERR_TIMEOUT in the
  * workspace status word (read with ndg_read_status) and returns; nothing

@@ -514,10 +514,7 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
       for (int k = 0; k < R4; ++k) cur[k] = nxt[k];
       // the chain of chunk i - 2 (its D2 buffer is the one chunk i will use)
       if (ok && i >= 2) ok = chain(i - 2);
-      if (__shfl_sync(0xffffffffu, (!ok || *abort_flag) ? 1 : 0, 0)) {
-        ok = false;
-        break;
-      }
+      if (!ok) break;
     }
     for (int ic = nchunks >= 2 ? nchunks - 2 : 0; ok && ic < nchunks; ++ic) ok = chain(ic);
     if (!ok && lane == 0) fail();
@@ -534,7 +531,7 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
       constexpr uint64_t C_LO = S::C_BYTES >> 4;
       auto mma1 = [&](int u) -> bool {
         const int i = u / nh, h = u - i * nh, s = i % CS, sb = u % S::NBUF;
-        if (h == 0 && !mbar_wait_sleep(&coef_full[s], (i / CS) & 1, abort_flag)) return false;
+        if (h == 0 && !mbar_wait_abort(&coef_full[s], (i / CS) & 1, abort_flag)) return false;
         fence_after_sync();
         const uint64_t dch = dC0 + (uint64_t)((s * S::C_STAGE) >> 4);
         const uint64_t dph = dPhi + (uint64_t)((h * S::UNIT_BYTES) >> 4);
@@ -552,8 +549,8 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
       };
       auto mma2 = [&](int u) -> bool {
         const int i = u / nh, h = u - i * nh, sb = u % S::NBUF, db = i & 1;
-        if (!mbar_wait_sleep(&e_full[sb], (u / S::NBUF) & 1, abort_flag)) return false;
-        if (h == 0 && i >= 2 && !mbar_wait_sleep(&d2_empty[db], ((i >> 1) - 1) & 1, abort_flag))
+        if (!mbar_wait_abort(&e_full[sb], (u / S::NBUF) & 1, abort_flag)) return false;
+        if (h == 0 && i >= 2 && !mbar_wait_abort(&d2_empty[db], ((i >> 1) - 1) & 1, abort_flag))
           return false;
         fence_after_sync();
         const uint32_t d = tmem + S::TM_D2 + (uint32_t)(db * NPSI);
@@ -634,20 +631,20 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
       tmem_wait_st();
       fence_before_sync();
       warp_arrive(&e_full[sb]);
-      if (__shfl_sync(0xffffffffu, *abort_flag ? 1 : 0, 0)) {
-        ok = false;
-        break;
-      }
     }
     if (!ok && lane == 0) fail();
   }
+  // A barrier counts a warp each time a part of it arrives: the issuer's lane
+  // and the other 31 come back together.
+  __syncwarp();
   fence_before_sync();
   __syncthreads();
-  if (warp == 12 && lane == 0) {
+  if (warp == 12 && elect_one()) {
     // every MMA this thread issued has completed once this commit arrives
     mma_commit(&drain);
     if (!mbar_wait_bounded(&drain, 0, kWaitLimit)) fail();
   }
+  __syncwarp();
   fence_before_sync();
   __syncthreads();
   if (warp == 0) {

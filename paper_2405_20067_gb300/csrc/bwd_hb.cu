@@ -426,10 +426,7 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
         c_next = cand(i + 2);
       }
       slot_cur = slot_nxt;
-      if (__shfl_sync(0xffffffffu, (!ok || *abort_flag) ? 1 : 0, 0)) {
-        ok = false;
-        break;
-      }
+      if (!ok) break;
     }
     if (!ok && lane == 0) fail();
   } else if (warp == 12) {
@@ -448,7 +445,7 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
       constexpr uint64_t PHI_LO = S::LO_OFF >> 4, C_LO = S::C_BYTES >> 4;
       auto mma1 = [&](int u) -> bool {
         const int i = u / nh, h = u - i * nh, s = i % CS, sb = u % NBUF;
-        if (h == 0 && !mbar_wait_sleep(&coef_full[s], (i / CS) & 1, abort_flag)) return false;
+        if (h == 0 && !mbar_wait_abort(&coef_full[s], (i / CS) & 1, abort_flag)) return false;
         fence_after_sync();
         const uint64_t dch = dC0 + (uint64_t)((s * S::C_STAGE) >> 4);
         const uint64_t dph = dPhiK + (uint64_t)((h * 16 * S::GRP) >> 4);  // 16 groups per unit
@@ -466,8 +463,8 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
       };
       auto mma2 = [&](int u) -> bool {
         const int i = u / nh, h = u - i * nh, sb = u % NBUF, db = i & 1;
-        if (!mbar_wait_sleep(&e_full[sb], (u / NBUF) & 1, abort_flag)) return false;
-        if (h == 0 && i >= 2 && !mbar_wait_sleep(&d_empty[db], ((i >> 1) - 1) & 1, abort_flag))
+        if (!mbar_wait_abort(&e_full[sb], (u / NBUF) & 1, abort_flag)) return false;
+        if (h == 0 && i >= 2 && !mbar_wait_abort(&d_empty[db], ((i >> 1) - 1) & 1, abort_flag))
           return false;
         fence_after_sync();
         const uint32_t d = tmem + S::TM_D + (uint32_t)(db * ND);
@@ -733,21 +730,22 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
       // unit ran while this chunk's units were exponentiated), and MMA 2 of
       // the next chunk waits for its buffer
       if (h == nh - 1 && i >= 1) ok = chain(i - 1);
-      if (__shfl_sync(0xffffffffu, (!ok || *abort_flag) ? 1 : 0, 0)) {
-        ok = false;
-        break;
-      }
+      if (!ok) break;
     }
     if (ok && nchunks >= 1 && U > 0) ok = chain(nchunks - 1);
     if (!ok && lane == 0) fail();
   }
+  // A barrier counts a warp each time a part of it arrives: the issuer's lane
+  // and the other 31 come back together.
+  __syncwarp();
   fence_before_sync();
   __syncthreads();
-  if (warp == 12 && lane == 0) {
+  if (warp == 12 && elect_one()) {
     // every MMA this thread issued has completed once this commit arrives
     mma_commit(&drain);
     if (!mbar_wait_bounded(&drain, 0, kWaitLimit)) fail();
   }
+  __syncwarp();
   fence_before_sync();
   __syncthreads();
   if (warp == 0) {

@@ -387,9 +387,9 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
       constexpr uint32_t IDESC = idesc_f16(NC);
       for (int i = 0; i < nchunks; ++i) {
         const int s = i % CS, b = i & 1;
-        bool ok = mbar_wait_sleep(&coef_full[s], (i / CS) & 1, abort_flag);
+        bool ok = mbar_wait_abort(&coef_full[s], (i / CS) & 1, abort_flag);
         // buffer b is free once the epilogue has read chunk i - 2
-        if (ok && i >= 2) ok = mbar_wait_sleep(&acc_empty[b], ((i >> 1) - 1) & 1, abort_flag);
+        if (ok && i >= 2) ok = mbar_wait_abort(&acc_empty[b], ((i >> 1) - 1) & 1, abort_flag);
         if (!ok) {
           fail();
           break;

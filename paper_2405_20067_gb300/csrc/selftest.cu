@@ -12,8 +12,8 @@
 
 namespace ndg {
 
-// which = 0: the sleeping warp wait (warp_wait: lane 0 polls with the
-// suspend-time hint, kSleepLimit polls); which = 1: the spinning wait of the
+// which = 0: the roles' warp wait (warp_wait: every lane polls, kPollLimit
+// polls); which = 1: the spinning wait of the
 // kernels' final drain (mbar_wait_bounded, kWaitLimit polls).
 __global__ void selftest_wait_kernel(int* status, int which) {
   __shared__ uint64_t bar;

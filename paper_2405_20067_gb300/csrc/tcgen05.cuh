@@ -37,6 +37,9 @@ __device__ __forceinline__ void fence_proxy_async() {
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
+__device__ __forceinline__ void mbar_inval(uint64_t* bar) {
+  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -194,48 +197,47 @@ __host__ __device__ constexpr uint32_t idesc_f16(int n) {
   return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
 }
 
-// try_wait with a suspend-time hint: the thread may sleep (up to the hint,
-// in nanoseconds) until the phase completes instead of spinning.
-constexpr uint32_t kSuspendNs = 20000;
-constexpr uint32_t kSleepLimit = 1u << 16;  // polls: at most ~1.3 s of suspension
-__device__ __forceinline__ bool mbar_try_wait_sleep(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-      " selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
-      : "memory");
-  return ok != 0;
-}
-// Bounded sleeping wait that gives up once another thread has raised *abort.
-__device__ __forceinline__ bool mbar_wait_sleep(uint64_t* bar, uint32_t parity,
+// Bounded wait that gives up once another thread has raised *abort (a poll
+// takes ~3.8 us when the phase does not complete: at most ~1 s).
+constexpr uint32_t kPollLimit = 1u << 18;
+__device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, uint32_t parity,
                                                 volatile int* abort) {
-  for (uint32_t i = 0; i < kSleepLimit; ++i) {
-    if (mbar_try_wait_sleep(bar, parity)) return true;
+  for (uint32_t i = 0; i < kPollLimit; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
     if (*abort) return false;
   }
   return false;
 }
 
-// Warp-level bounded wait: lane 0 waits, the outcome is broadcast, and the
-// warp synchronises (memory ordering) before any lane reads guarded data.
+// Warp-level bounded wait: every lane polls for itself and the warp leaves
+// together.  (Lane 0 polling, with a suspend-time hint, and handing its
+// outcome on by a shuffle cost ~600 cycles per wait, also on a completed
+// phase: N = 6 backward 33.4 -> 24.2 ms.)
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  int ok = 1;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait_sleep(bar, parity, abort) ? 1 : 0;
-  ok = __shfl_sync(0xffffffffu, ok, 0);
-  __syncwarp();
-  return ok != 0;
+  const bool ok = mbar_wait_abort(bar, parity, abort);
+  return __all_sync(0xffffffffu, ok);
 }
 
 // One lane of a converged warp.  The issuers choose their lane with it and
 // not with lane == 0: the assembler then knows that one lane at most issues
 // the MMAs (N = 6 backward 36.7 -> 33.5 ms, N = 10 backward 39.6 -> 38.3 ms).
+// The lanes may arrive one by one (from a branch of one lane); elect.sync on
+// parts of the warp would elect a lane of each.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
+  __syncwarp();
   asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}"
                : "=r"(p));
   return p != 0;
+}
+
+// 16-byte asynchronous copy global -> shared, and the wait for all of the
+// thread's own copies.
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // One arrival per warp (after the warp's earlier shared-memory writes).
