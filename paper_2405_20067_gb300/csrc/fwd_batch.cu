@@ -10,16 +10,22 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
   return v;
 }
 
+// One function per N, not inlined: the register allocation of one N's tile
+// code then does not depend on the eleven others' (inlined, addresses of all
+// of them were kept live and spilled).
+template <int N>
+__device__ __noinline__ void fwd_tile_fn(const FwdArgs* args, long long t) {
+  const FwdArgs a = *args;
+  fwd_tile<N>(a, t);
+}
+
 // Persistent CTAs (one per SM) over the (frame, tile) work list of a batch
 // of frames of any N <= 12: a CTA takes the next item with an atomic
 // cursor, renders that tile with fwd_tile<N> of the item's frame (so a
 // frame's outputs equal those of its own fwd_h_kernel launch), and the CTA
 // that completes a frame's last tile stamps the frame's completion time.
 // Tensor memory is allocated once per CTA and reused by every tile.
-__global__ void __launch_bounds__(416, 1) fwd_h_batch_kernel(FwdBatchArgs b) {
-  extern __shared__ __align__(128) uint8_t dsm[];
-  uint8_t* base = (uint8_t*)(((uintptr_t)dsm + 127) & ~(uintptr_t)127);
-  __shared__ FwdHSync sy;
+__global__ void __launch_bounds__(kFwdThreads, 1) fwd_h_batch_kernel(FwdBatchArgs b) {
   __shared__ long long s_item;
   __shared__ int s_stop;
   const int tid = threadIdx.x;
@@ -28,7 +34,7 @@ __global__ void __launch_bounds__(416, 1) fwd_h_batch_kernel(FwdBatchArgs b) {
     if (b.stamps) atomicMin(&b.stamps[0], globaltimer_ns());
   }
   if (tid < 32) {
-    tmem_alloc(&sy.tmem_base, 512);
+    tmem_alloc(&fwd_sync().tmem_base, 512);
     tmem_relinquish();
   }
   for (;;) {
@@ -44,25 +50,24 @@ __global__ void __launch_bounds__(416, 1) fwd_h_batch_kernel(FwdBatchArgs b) {
       if (b.tile_start[mid] <= item) f = mid;
       else hi = mid - 1;
     }
-    const FwdArgs a = b.frames[f];
     const long long t = item - b.tile_start[f];
     switch (b.N[f]) {
-      case 1: fwd_tile<1>(a, t, base, sy); break;
-      case 2: fwd_tile<2>(a, t, base, sy); break;
-      case 3: fwd_tile<3>(a, t, base, sy); break;
-      case 4: fwd_tile<4>(a, t, base, sy); break;
-      case 5: fwd_tile<5>(a, t, base, sy); break;
-      case 6: fwd_tile<6>(a, t, base, sy); break;
-      case 7: fwd_tile<7>(a, t, base, sy); break;
-      case 8: fwd_tile<8>(a, t, base, sy); break;
-      case 9: fwd_tile<9>(a, t, base, sy); break;
-      case 10: fwd_tile<10>(a, t, base, sy); break;
-      case 11: fwd_tile<11>(a, t, base, sy); break;
-      case 12: fwd_tile<12>(a, t, base, sy); break;
+      case 1: fwd_tile_fn<1>(b.frames + f, t); break;
+      case 2: fwd_tile_fn<2>(b.frames + f, t); break;
+      case 3: fwd_tile_fn<3>(b.frames + f, t); break;
+      case 4: fwd_tile_fn<4>(b.frames + f, t); break;
+      case 5: fwd_tile_fn<5>(b.frames + f, t); break;
+      case 6: fwd_tile_fn<6>(b.frames + f, t); break;
+      case 7: fwd_tile_fn<7>(b.frames + f, t); break;
+      case 8: fwd_tile_fn<8>(b.frames + f, t); break;
+      case 9: fwd_tile_fn<9>(b.frames + f, t); break;
+      case 10: fwd_tile_fn<10>(b.frames + f, t); break;
+      case 11: fwd_tile_fn<11>(b.frames + f, t); break;
+      case 12: fwd_tile_fn<12>(b.frames + f, t); break;
       default: break;  // the host admits 1 <= N <= 12 only
     }
     if (tid == 0) {
-      if (sy.s_abort) s_stop = 1;  // a timed-out wait: take no further items
+      if (fwd_sync().s_abort) s_stop = 1;  // a timed-out wait: take no further items
       __threadfence();
       const unsigned long long nt = (unsigned long long)(b.tile_start[f + 1] - b.tile_start[f]);
       if (atomicAdd(&b.done[f], 1ull) + 1ull == nt && b.stamps) b.stamps[1 + f] = globaltimer_ns();
@@ -70,14 +75,14 @@ __global__ void __launch_bounds__(416, 1) fwd_h_batch_kernel(FwdBatchArgs b) {
   }
   if (tid < 32) {
     fence_after_sync();
-    tmem_dealloc(sy.tmem_base, 512);
+    tmem_dealloc(fwd_sync().tmem_base, 512);
   }
 }
 
 int launch_fwd_tc_batch(const FwdBatchArgs& b, unsigned smem, int grid, cudaStream_t s) {
   if (b.n_items <= 0 || grid <= 0) return 0;
   cudaFuncSetAttribute(fwd_h_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  fwd_h_batch_kernel<<<(unsigned)grid, 416, smem, s>>>(b);
+  fwd_h_batch_kernel<<<(unsigned)grid, kFwdThreads, smem, s>>>(b);
   return 1;
 }
 

@@ -6,20 +6,17 @@ namespace ndg {
 
 // One CTA per tile (a tile list selects a subset; surplus CTAs leave at once).
 template <int N>
-__global__ void __launch_bounds__(416, 1) fwd_h_kernel(FwdArgs a) {
-  extern __shared__ __align__(128) uint8_t dsm[];
-  uint8_t* base = (uint8_t*)(((uintptr_t)dsm + 127) & ~(uintptr_t)127);
-  __shared__ FwdHSync sy;
+__global__ void __launch_bounds__(kFwdThreads, 1) fwd_h_kernel(FwdArgs a) {
   if (a.tiles && (int)blockIdx.x >= *a.n_tiles) return;
   const long long t = a.tiles ? (long long)a.tiles[blockIdx.x] : (long long)blockIdx.x;
   if (threadIdx.x < 32) {
-    tmem_alloc(&sy.tmem_base, 512);
+    tmem_alloc(&fwd_sync().tmem_base, 512);
     tmem_relinquish();
   }
-  fwd_tile<N>(a, t, base, sy);
+  fwd_tile<N>(a, t);
   if (threadIdx.x < 32) {
     fence_after_sync();
-    tmem_dealloc(sy.tmem_base, 512);
+    tmem_dealloc(fwd_sync().tmem_base, 512);
   }
 }
 
@@ -42,7 +39,7 @@ int launch_fwd_tc(int N, const FwdArgs& a, long long T, cudaStream_t s) {
   {                                                                                     \
     cudaFuncSetAttribute(fwd_h_kernel<n>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
                          (int)FwdHShape<n>::SMEM);                                      \
-    fwd_h_kernel<n><<<(unsigned)T, 416, FwdHShape<n>::SMEM, s>>>(a);                    \
+    fwd_h_kernel<n><<<(unsigned)T, kFwdThreads, FwdHShape<n>::SMEM, s>>>(a);                    \
   }
   switch (N) {
     NDG_H_CASE(1, L_H) NDG_H_CASE(2, L_H) NDG_H_CASE(3, L_H) NDG_H_CASE(4, L_H)

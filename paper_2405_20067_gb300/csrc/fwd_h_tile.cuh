@@ -17,32 +17,44 @@
 //     stage carries a flag so that chunks without such rows skip it).
 //
 // CTA = one tile of up to 256 queries (two M = 128 row blocks sharing the
-// candidate operand), 416 threads, one CTA per SM.  What bounds the tile is
-// the shared-memory pipe, which the MMAs' operand reads (one wavefront per
-// 128 bytes), the weight loads and the coefficient rows share; it was 68%
-// (N = 6) to 82% (N = 10) busy, and every barrier or load behind it waited
-// ~400 cycles, while Phi was an operand in shared memory and each weight
-// load served four query rows.  So Phi, the same for all of a tile's chunks,
-// is the A operand in tensor memory (hi and lo; N >= 10 has room for hi only
-// and keeps lo in shared memory), the chunks are of 96 candidates so that two
-// double-buffered accumulators and Phi share the 512 columns (an MMA of 96
-// columns costs its share of one of 128), and a weight load serves eight rows.
-// Measured: N = 10 480 x 272 frame (100,000 Gaussians) 6.78 -> 6.00 ms, N = 10
-// fit 14.6 -> 12.6 ms, N = 8 5,000 Gaussians 159 -> 136 us.
-//   warps 0-3   builders: a warp turns its 32 candidates of a chunk into
+// candidate operand), 544 threads (96 registers), one CTA per SM.  What bounds
+// the tile: at N = 6 the epilogue's chain of exponentials and colour sums, at
+// N = 10 the builders and the MMAs (30 of 48 cycles per chunk).  What the
+// layout answers to:
+//   * the shared-memory pipe, shared by the MMAs' operand reads (a wavefront
+//     per 128 bytes), the weight loads and the coefficient rows, was 68%
+//     (N = 6) to 82% (N = 10) busy with Phi as a shared-memory operand.  Phi,
+//     the same for all of a tile's chunks, is the A operand in tensor memory
+//     (hi and lo; N >= 10 has room for hi only and keeps lo in shared memory),
+//     and the chunks are of 96 candidates so that two double-buffered
+//     accumulators and Phi share the 512 columns (an MMA of 96 columns costs
+//     its share of one of 128);
+//   * one builder warp per SM sub-partition issued an instruction every four
+//     cycles and waited for its own record loads: eight builder warps (six at
+//     N = 12), records by cp.async a group ahead, consecutive lanes copying
+//     consecutive parts of a record;
+//   * MUFU and FMA took turns inside an epilogue warp: the exponentials of 16
+//     columns are issued with the sums of the 16 before.
+// Measured, kernel alone: N = 6 256 x 256 frame (10,000 Gaussians) 235 -> 178
+// us, N = 8 701 x 397 (60,000) 5.72 -> 4.20 ms, N = 10 480 x 272 (100,000)
+// 6.79 -> 5.62 ms, N = 10 1080p (500,000) 491 -> 410 ms, N = 12 evaluation
+// (10,000, 32,768 queries) 303 -> 233 us.  Four builders with 13 warps and
+// eight rows per weight load measured 124 us where this takes 112 (N = 8,
+// 5,000 Gaussians; 159 at first).
+//   warps 0-7   builders: a warp turns its 32 candidates of a chunk into
 //               coefficient rows (FP16 hi / lo, K-major no-swizzle layout)
 //               and weight pair entries in one of CS shared-memory stages
 //               and arrives on coef_full;
-//   warp 12     MMA issuer: one lane issues the MMAs of chunk i once its
-//               stage is full and accumulator buffer i & 1 is free, and
-//               commits them to acc_full and coef_empty (a warp of its own,
-//               so that issuing overlaps the building of the next chunks);
-//   warps 4-11  epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 of both
-//               row blocks at half of the chunk's columns with the 16x256b
-//               load shape (a thread holds 4 rows x 2 columns of every
-//               8-column group); it forms e = 2^s and accumulates w e; row
-//               sums are completed with shuffles and, over the two column
-//               halves, through shared memory at the end.
+//   warps 8-15  epilogue: warps 8-11 serve row block 0, 12-15 row block 1;
+//               warp w reads TMEM lanes 32 (w % 4) .. + 31 of its block with
+//               the 16x256b load shape (a thread holds 4 rows x 2 columns of
+//               every 8-column group, so each weight load serves four rows),
+//               forms e = 2^s and accumulates w e; row sums are completed
+//               with shuffles at the end;
+//   warp 16     MMA issuer: one lane issues the MMAs of a row block of chunk i
+//               once its stage is full and that block of accumulator buffer
+//               i & 1 is free, commits them to acc_full and, after both
+//               blocks, to coef_empty.
 // Barrier operations are one per warp (an elected lane), and every wait is
 // bounded: on a timeout the kernel records NDG_ERR_TIMEOUT, lets the issued
 // MMAs finish (bounded), frees its tensor memory and returns.
@@ -56,6 +68,26 @@
 #include "tcgen05.cuh"
 
 namespace ndg {
+
+// Warps of the forward's CTA: builders, epilogue, issuer.
+constexpr int kFwdBuilders = 8;
+constexpr int kFwdEpi0 = kFwdBuilders, kFwdIssuer = kFwdBuilders + 8;
+constexpr int kFwdThreads = 32 * (kFwdIssuer + 1);
+
+// Barriers and small shared state of one tile, sized for the largest shape
+// (CS <= 4 coefficient stages, N <= 12).
+struct FwdHSync {
+  // accumulator barriers per (buffer, row block): index 2 b + h
+  uint64_t coef_full[4], coef_empty[4], acc_full[4], acc_empty[4], drain;
+  static constexpr int kBarriers = 17;
+  uint32_t tmem_base;
+  float sred[8 * 12 * 2];
+  float sctr[12], sh[12];
+  __align__(16) int sflag[4][4];  // per stage and 32-candidate group: a row was scaled
+  int s_abort;
+};
+
+static_assert(sizeof(FwdHSync) <= 1536, "static shared memory");
 
 template <int N>
 struct FwdHShape {
@@ -80,14 +112,16 @@ struct FwdHShape {
   // coefficient stages: as many as fit next to Phi (at most 4; 2 KB are left
   // for the static shared variables).  The builders run up to CS chunks ahead
   // of the epilogue, which frees a stage only at the end of its chunk.
-  static constexpr uint32_t STAGE_ROOM = 227u * 1024u - 2048u - PHI_BYTES - 128u;
+  static constexpr uint32_t REC_STRIDE = (R / 4) | 1;  // float4s: odd, so that lanes' rows miss no bank
+  static constexpr int BW = N <= 11 ? kFwdBuilders : 6;  // builder warps with room for their records
+  static constexpr uint32_t REC_BYTES = (uint32_t)BW * 32 * REC_STRIDE * 16;  // a group of records per builder warp
+  static constexpr uint32_t STAGE_ROOM = 227u * 1024u - 2048u - PHI_BYTES - REC_BYTES - 128u;
   static constexpr int CS = STAGE_ROOM / C_STAGE >= 4 ? 4 : (int)(STAGE_ROOM / C_STAGE);
-  static constexpr uint32_t SMEM_USED = PHI_BYTES + CS * C_STAGE + 128;
+  static constexpr uint32_t SMEM_USED = PHI_BYTES + CS * C_STAGE + REC_BYTES + 128;
   // more than half of the SM's shared memory: one CTA per SM
   static constexpr uint32_t SMEM = SMEM_USED > 116u * 1024u ? SMEM_USED : 116u * 1024u;
-  static_assert(SMEM <= 227u * 1024u, "shared memory");
+  static_assert(SMEM + 2048 <= 227u * 1024u, "shared memory");  // 2 KB: static variables
   static_assert(CS >= 2, "coefficient stages");
-  static_assert(2 * B_BYTES >= 256 * 12, "row sums of the second column half");
 };
 
 namespace {
@@ -112,29 +146,29 @@ constexpr float kRowMax = 16384.0f;  // coefficient rows are kept below 2^14 (FP
 
 }  // namespace
 
-// Barriers and small shared state of one tile, sized for the largest shape
-// (CS <= 4 coefficient stages, N <= 12).
-struct FwdHSync {
-  uint64_t coef_full[4], coef_empty[4], acc_full[2], acc_empty[2], drain;
-  uint32_t tmem_base;
-  float sred[8 * 12 * 2];
-  float sctr[12], sh[12];
-  __align__(16) int sflag[4][4];  // per stage and 32-candidate group: a row was scaled
-  int s_abort;
-};
+// The CTA's barriers and small shared state, and its dynamic shared memory
+// (no rounding of its address: the alignment is declared, and every offset
+// then is a constant).
+static __shared__ FwdHSync s_fwd;
+__device__ __forceinline__ FwdHSync& fwd_sync() { return s_fwd; }
+__device__ __forceinline__ uint8_t* fwd_smem() {
+  extern __shared__ __align__(1024) uint8_t dsm[];
+  return dsm;
+}
 
 // Query tile t on the tensor cores, by the whole CTA.  The caller owns the
-// tensor memory (all 512 columns, address in sy.tmem_base, visible after
-// the tile's first block barrier).  Returns after a block barrier with every
-// MMA of the tile complete, so that the caller may start another tile.
+// tensor memory (all 512 columns, address in fwd_sync().tmem_base, visible
+// after the tile's first block barrier).  Returns after a block barrier with
+// every MMA of the tile complete, so that the caller may start another tile.
 template <int N>
-__device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t* base,
-                                         FwdHSync& sy) {
+__device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t) {
   using S = FwdHShape<N>;
   constexpr int P = S::P, KP = S::KP, NC = S::NC, CS = S::CS, R = S::R, R4 = R / 4;
   static_assert(CS <= 4 && N <= 12, "FwdHSync sizes");
-  uint8_t* Alo = base;                // Phi lo, where tensor memory does not hold it
+  FwdHSync& sy = fwd_sync();
+  uint8_t* Alo = fwd_smem();  // Phi lo, where tensor memory does not hold it
   uint8_t* Cst = Alo + S::PHI_BYTES;  // CS stages of (Bhi, Blo, weights)
+  uint8_t* Rec = Cst + CS * S::C_STAGE;  // 32 records per builder warp
   uint64_t* coef_full = sy.coef_full;
   uint64_t* coef_empty = sy.coef_empty;
   uint64_t* acc_full = sy.acc_full;
@@ -153,20 +187,20 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
 
   // ---- setup: barriers, tile centre and scales, Phi rows (epilogue warps)
   if (tid == 0) {
-    for (int i = 0; i < CS; ++i) {
+    for (int i = 0; i < 4; ++i) {
       mbar_init(&coef_full[i], S::GPC);
-      mbar_init(&coef_empty[i], 1 + 8);  // issuer commit + the epilogue warps
+      mbar_init(&coef_empty[i], 1 + 4 * nh);  // issuer commit + the busy epilogue warps
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&acc_full[i], 1);
-      mbar_init(&acc_empty[i], 8);
+    for (int i = 0; i < 4; ++i) {
+      mbar_init(&acc_full[i], 2);  // issuer commit and arrival
+      mbar_init(&acc_empty[i], 4);
     }
     mbar_init(&drain, 1);
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  const int row = tid - 128;  // epilogue threads: Phi row
-  const bool is_epi = warp >= 4 && warp < 12;
+  const int row = tid - 32 * kFwdEpi0;  // epilogue threads: Phi row
+  const bool is_epi = warp >= kFwdEpi0 && warp < kFwdIssuer;
   const bool active_row = is_epi && row < nq;
   float xq[N];
 #pragma unroll
@@ -181,8 +215,8 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
         hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
       }
       if (lane == 0) {
-        sred[((warp - 4) * N + d) * 2] = lo;
-        sred[((warp - 4) * N + d) * 2 + 1] = hi;
+        sred[((warp - kFwdEpi0) * N + d) * 2] = lo;
+        sred[((warp - kFwdEpi0) * N + d) * 2 + 1] = hi;
       }
     }
   }
@@ -212,9 +246,9 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
     phi[P + N] = active_row ? 1.0f : 0.0f;
 #pragma unroll
     for (int k = P + N + 1; k < KP; ++k) phi[k] = 0.0f;
-    // row `row` = lane 32 (warp % 4) + lane of row block (warp - 4) / 4
+    // row `row` = lane 32 (warp % 4) + lane of its row block
     const uint32_t ph = sy.tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + S::TM_PHI +
-                        (uint32_t)(((warp - 4) >> 2) * (KP / 2));
+                        (uint32_t)(((warp - kFwdEpi0) >> 2) * (KP / 2));
     fence_after_sync();
 #pragma unroll
     for (int k = 0; k < KP; k += 8) {
@@ -242,98 +276,140 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
     if (a.status) set_status(a.status, NDG_ERR_TIMEOUT);
   };
 
-  // epilogue warps 4-7: the thread's query row inside each row block, and its
-  // rows' sums
-  const int my_row = (warp & 3) * 32 + ((lane & 3) >> 1) * 16 + (lane & 1) * 8 + (lane >> 2);
-  float rs[2][3] = {};
-
-  if (warp < 4) {
+  if (warp < S::BW) {
     // ---- builders
-    // warp w builds the 32-candidate groups w, w + 4, ...; group g is rows
+    // warp w builds the 32-candidate groups w, w + BW, ...; group g is rows
     // 32 (g % GPC) .. + 31 of chunk g / GPC
     const int ngroups = nchunks * S::GPC;
-    float hsc[N];
-#pragma unroll
-    for (int d = 0; d < N; ++d) hsc[d] = sh[d];
     auto cand = [&](int gr) -> int {
       const long long c = beg + (long long)gr * 32 + lane;
       const int g = c < end ? a.ids[c] : -1;
       return ((unsigned)g < (unsigned)a.Ge) ? g : -1;
     };
     const int stride4 = a.rec_stride4 > 0 ? a.rec_stride4 : R4;
-    auto load = [&](int g, float4 (&r)[R4]) {
-      if (g >= 0) {
-        const float4* src = reinterpret_cast<const float4*>(a.rec) + (size_t)g * stride4;
+    // The records of a group come by asynchronous copies into the warp's 32
+    // rows, issued as soon as the group before has been read into registers,
+    // and arrive while that group is built.  Consecutive lanes copy
+    // consecutive 16-byte parts of a record: one lane per record would take
+    // 32 cache lines an instruction.
+    float4* rows = reinterpret_cast<float4*>(Rec) + (size_t)warp * 32 * S::REC_STRIDE;
+    auto fetch = [&](int g) {
 #pragma unroll
-        for (int k = 0; k < R4; ++k) r[k] = __ldg(src + k);
-      } else {
-#pragma unroll
-        for (int k = 0; k < R4; ++k) r[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k = 0; k < R4; ++k) {
+        const int r = (k * 32 + lane) / R4, part = k * 32 + lane - r * R4;
+        const int gr = __shfl_sync(0xffffffffu, g, r);
+        if (gr >= 0)
+          cp_async16(rows + r * S::REC_STRIDE + part,
+                     reinterpret_cast<const float4*>(a.rec) + (size_t)gr * stride4 + part);
       }
     };
-    // N <= 6: the records of the warp's next group are loaded into registers
-    // while a group is built; larger records are loaded right after a build (the
-    // latency overlaps the next stage wait) to keep the register count down.
-    constexpr bool PRE = N <= 6;
-    float4 cur[R4], nxt[PRE ? R4 : 1];
-    load(cand(warp), cur);
-    int g_next = cand(warp + 4);
-    for (int gr = warp; gr < ngroups; gr += 4) {
+    int g_cur = cand(warp), g_next = cand(warp + S::BW);
+    fetch(warp < ngroups ? g_cur : -1);
+    for (int gr = warp; gr < ngroups; gr += S::BW) {
       const int i = gr / S::GPC, s = i % CS;
       const int j = (gr - i * S::GPC) * 32 + lane;
-      if constexpr (PRE) {
-        load(g_next, nxt);  // the warp's next group (zeros past the end)
-        g_next = cand(gr + 8);
-      }
       bool ok = true;
-      if (i >= CS) ok = warp_wait(&coef_empty[s], ((i / CS) - 1) & 1, abort_flag);
+      cp_async_wait_all();
+      __syncwarp();
+      // N >= 9: the record stays in its row and is read twice (112 to 200 of
+      // a thread's 96 registers' worth would be spilled otherwise); smaller
+      // ones are read into registers and the next group's copies start at once.
+      constexpr bool STREAM = N >= 9;
+      float4* mine = rows + lane * S::REC_STRIDE;
+      if (g_cur < 0) {
+#pragma unroll
+        for (int k = 0; k < R4; ++k) mine[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      float buf[STREAM ? 4 : R];
+      if constexpr (!STREAM) {
+#pragma unroll
+        for (int k = 0; k < R4; ++k) {
+          const float4 r = mine[k];
+          buf[4 * k] = r.x; buf[4 * k + 1] = r.y; buf[4 * k + 2] = r.z; buf[4 * k + 3] = r.w;
+        }
+        __syncwarp();  // every lane has its row: the next group's may land
+        fetch(g_next);
+        g_cur = g_next;
+        g_next = cand(gr + 2 * S::BW);
+      }
+      if (ok && i >= CS) ok = warp_wait(&coef_empty[s], ((i / CS) - 1) & 1, abort_flag);
       if (!ok && lane == 0) fail();
       uint8_t* st = Cst + s * S::C_STAGE;
       bool scaled = false;
       if (ok) {
-        float buf[R];
-#pragma unroll
-        for (int k = 0; k < R4; ++k) {
-          buf[4 * k] = cur[k].x; buf[4 * k + 1] = cur[k].y;
-          buf[4 * k + 2] = cur[k].z; buf[4 * k + 3] = cur[k].w;
-        }
-        float mt[N], tA[N];
-#pragma unroll
-        for (int d = 0; d < N; ++d) mt[d] = buf[P + d] - sctr[d];
-        float cst = 0.0f;
-#pragma unroll
-        for (int d = 0; d < N; ++d) {
-          float s2 = 0.0f;
-#pragma unroll
-          for (int k = 0; k < N; ++k) s2 = fmaf(buf[d >= k ? tri(d) + k : tri(k) + d], mt[k], s2);
-          tA[d] = s2;
-          cst = fmaf(mt[d], s2, cst);
-        }
-        // coefficients kb .. kb + 7 (kb compile-time after unrolling):
-        // quadratic (d, e), linear d, constant, zero padding
-        auto cblock = [&](int kb, float (&v)[8]) {
-#pragma unroll
-          for (int q = 0; q < 8; ++q) v[q] = 0.0f;
-#pragma unroll
-          for (int d = 0; d < N; ++d)
-#pragma unroll
-            for (int e2 = 0; e2 <= d; ++e2) {
-              const int p = tri(d) + e2;
-              if (p >= kb && p < kb + 8)
-                v[p - kb] = kNegHalfLog2eH * (d == e2 ? buf[p] : 2.0f * buf[p]) * (hsc[d] * hsc[e2]);
-            }
-#pragma unroll
-          for (int d = 0; d < N; ++d)
-            if (P + d >= kb && P + d < kb + 8) v[P + d - kb] = (kNegHalfLog2eH * -2.0f) * tA[d] * hsc[d];
-          if (P + N >= kb && P + N < kb + 8) v[P + N - kb] = kNegHalfLog2eH * cst;
+        float mt[N], tA[N], cst = 0.0f, mx = 0.0f;
+        float cf[STREAM ? 8 : KP];
+        float wc[3];
+        // coefficient of the quadratic term (d, e), e <= d, from A_de
+        auto quad_coef = [&](float av, int d, int e2) {
+          const float kd = kNegHalfLog2eH * sh[d];
+          return av * (d == e2 ? kd : 2.0f * kd) * sh[e2];
         };
-        float mx = 0.0f;
+        if constexpr (STREAM) {
 #pragma unroll
-        for (int kb = 0; kb < KP; kb += 8) {
-          float v[8];
-          cblock(kb, v);
+          for (int k = P / 4; k < R4; ++k) {
+            const float4 q = mine[k];
+            const float qa[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-          for (int q = 0; q < 8; ++q) mx = fmaxf(mx, fabsf(v[q]));
+            for (int c = 0; c < 4; ++c) {
+              const int p = 4 * k + c - P;
+              if (p >= 0 && p < N) mt[p] = qa[c] - sctr[p];
+              if (p >= N && p < N + 3) wc[p - N] = qa[c];
+            }
+          }
+#pragma unroll
+          for (int d = 0; d < N; ++d) tA[d] = 0.0f;
+          // A m~, every sum in the order of the products' second index, as below
+#pragma unroll
+          for (int k = 0; 4 * k < P; ++k) {
+            const float4 q = mine[k];
+            const float qa[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+              for (int d = 0; d < N; ++d) {
+                const int e2 = 4 * k + c - tri(d);
+                if (e2 >= 0 && e2 <= d) {
+                  tA[d] = fmaf(qa[c], mt[e2], tA[d]);
+                  if (e2 < d) tA[e2] = fmaf(qa[c], mt[d], tA[e2]);
+                  mx = fmaxf(mx, fabsf(quad_coef(qa[c], d, e2)));
+                }
+              }
+          }
+#pragma unroll
+          for (int d = 0; d < N; ++d) cst = fmaf(mt[d], tA[d], cst);
+#pragma unroll
+          for (int d = 0; d < N; ++d) {
+            tA[d] = (-2.0f * (kNegHalfLog2eH * sh[d])) * tA[d];
+            mx = fmaxf(mx, fabsf(tA[d]));
+          }
+          cst *= kNegHalfLog2eH;
+          mx = fmaxf(mx, fabsf(cst));
+        } else {
+#pragma unroll
+          for (int d = 0; d < N; ++d) mt[d] = buf[P + d] - sctr[d];
+#pragma unroll
+          for (int d = 0; d < N; ++d) {
+            float s2 = 0.0f;
+#pragma unroll
+            for (int k = 0; k < N; ++k) s2 = fmaf(buf[d >= k ? tri(d) + k : tri(k) + d], mt[k], s2);
+            tA[d] = s2;
+            cst = fmaf(mt[d], s2, cst);
+          }
+          // the coefficients, in the record's place (the scales are powers of
+          // two, so their order does not change a bit): quadratic (d, e),
+          // linear d, constant, zero padding
+#pragma unroll
+          for (int d = 0; d < N; ++d) {
+#pragma unroll
+            for (int e2 = 0; e2 <= d; ++e2) cf[tri(d) + e2] = quad_coef(buf[tri(d) + e2], d, e2);
+            cf[P + d] = (-2.0f * (kNegHalfLog2eH * sh[d])) * tA[d];
+          }
+          cf[P + N] = kNegHalfLog2eH * cst;
+#pragma unroll
+          for (int k = P + N + 1; k < KP; ++k) cf[k] = 0.0f;
+#pragma unroll
+          for (int k = 0; k <= P + N; ++k) mx = fmaxf(mx, fabsf(cf[k]));
         }
         float back = 1.0f, down = 1.0f;
         if (mx > kRowMax) {  // divide the row by 2^e, e = exponent(mx) - 13
@@ -342,42 +418,65 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
           down = __uint_as_float((uint32_t)(127 - e) << 23);
           back = __uint_as_float((uint32_t)(127 + e) << 23);
           scaled = true;
+          if constexpr (!STREAM) {
+#pragma unroll
+            for (int k = 0; k <= P + N; ++k) cf[k] *= down;
+          }
         }
+        if constexpr (STREAM) asm volatile("" ::: "memory");  // read the row again
 #pragma unroll
         for (int kb = 0; kb < KP; kb += 8) {
-          float v[8];
-          cblock(kb, v);
+          if constexpr (STREAM) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) cf[q] = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              if (kb + 4 * k >= P) continue;
+              const float4 q = mine[kb / 4 + k];
+              const float qa[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int d = 0; d < N; ++d) {
+                  const int e2 = kb + 4 * k + c - tri(d);
+                  if (e2 >= 0 && e2 <= d) cf[4 * k + c] = quad_coef(qa[c], d, e2) * down;
+                }
+            }
+#pragma unroll
+            for (int d = 0; d < N; ++d)
+              if (P + d >= kb && P + d < kb + 8) cf[P + d - kb] = tA[d] * down;
+            if (P + N >= kb && P + N < kb + 8) cf[P + N - kb] = cst * down;
+          }
+          const float* c = STREAM ? cf : cf + kb;
           uint4 h, l;
-          split_h2(v[0] * down, v[1] * down, h.x, l.x);
-          split_h2(v[2] * down, v[3] * down, h.y, l.y);
-          split_h2(v[4] * down, v[5] * down, h.z, l.z);
-          split_h2(v[6] * down, v[7] * down, h.w, l.w);
+          split_h2(c[0], c[1], h.x, l.x);
+          split_h2(c[2], c[3], h.y, l.y);
+          split_h2(c[4], c[5], h.z, l.z);
+          split_h2(c[6], c[7], h.w, l.w);
           const uint32_t off = kmajor_off_h(j, kb, S::SBO);
           *reinterpret_cast<uint4*>(st + off) = h;
           *reinterpret_cast<uint4*>(st + S::B_BYTES + off) = l;
         }
         float* wd = reinterpret_cast<float*>(st + 2 * S::B_BYTES) + (j >> 1) * 8 + (j & 1);
-        wd[0] = buf[P + N];
-        wd[2] = buf[P + N + 1];
-        wd[4] = buf[P + N + 2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) wd[2 * c] = STREAM ? wc[c] : buf[STREAM ? 0 : P + N + c];
         wd[6] = back;
       }
       const bool any_scaled = __any_sync(0xffffffffu, scaled);
       if (lane == 0) sflag[s][gr - i * S::GPC] = any_scaled ? 1 : 0;
       fence_proxy_async();
       warp_arrive(&coef_full[s]);
-      if constexpr (PRE) {
-#pragma unroll
-        for (int k = 0; k < R4; ++k) cur[k] = nxt[k];
-      }
       // a CTA that gives up stops every role at its next blocked wait
       if (!ok) break;
-      if constexpr (!PRE) {
-        load(g_next, cur);  // the warp's next group
-        g_next = cand(gr + 8);
+      if constexpr (STREAM) {
+        __syncwarp();
+        fetch(g_next);
+        g_cur = g_next;
+        g_next = cand(gr + 2 * S::BW);
       }
     }
-  } else if (warp == 12) {
+    cp_async_wait_all();
+  } else if (warp == kFwdIssuer) {
     // ---- MMA issuer
     if (elect_one()) {
       // descriptor bases (a descriptor for base + off is base + off / 16)
@@ -388,15 +487,12 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
       for (int i = 0; i < nchunks; ++i) {
         const int s = i % CS, b = i & 1;
         bool ok = mbar_wait_abort(&coef_full[s], (i / CS) & 1, abort_flag);
-        // buffer b is free once the epilogue has read chunk i - 2
-        if (ok && i >= 2) ok = mbar_wait_abort(&acc_empty[b], ((i >> 1) - 1) & 1, abort_flag);
-        if (!ok) {
-          fail();
-          break;
-        }
-        fence_after_sync();
         const uint64_t dbh = dB0 + (uint64_t)((s * S::C_STAGE) >> 4);
-        for (int h = 0; h < nh; ++h) {
+        for (int h = 0; ok && h < nh; ++h) {
+          // row block h of buffer b is free once its epilogue group has read chunk i - 2
+          if (i >= 2) ok = mbar_wait_abort(&acc_empty[2 * b + h], ((i >> 1) - 1) & 1, abort_flag);
+          if (!ok) break;
+          fence_after_sync();
           const uint32_t d = tmem + (uint32_t)((2 * b + h) * NC);
           const uint32_t ah = tmem + S::TM_PHI + (uint32_t)(h * (KP / 2));
           const uint64_t dal = dA0 + (uint64_t)((h * S::HALF_BYTES) >> 4);
@@ -408,156 +504,148 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t, uint8_t*
             if constexpr (S::LO_TM) mma_f16_ts(d, ah + KP + 8u * ks, dbh + ko, IDESC, 1u);
             else mma_f16(d, dal + ko, dbh + ko, IDESC, 1u);
           }
+          mma_commit(&acc_full[2 * b + h]);
+          mbar_arrive(&acc_full[2 * b + h]);  // after coef_full: hands the weights on to the epilogue
         }
-        mma_commit(&acc_full[b]);
+        if (!ok) {
+          fail();
+          break;
+        }
         mma_commit(&coef_empty[s]);
       }
     }
-  } else {
+  } else if (is_epi) {
     // ---- epilogue (tcgen05.ld 16x256b: thread t holds lanes t/4 and t/4 + 8
     // of a 16-lane half at columns 2 (t % 4) + {0, 1} of every 8-column group).
-    // The warp takes its 32 lanes of both row blocks, so that one load of a
-    // pair of weights serves eight query rows.
-    constexpr int CW = NC / 2, NB = CW / 16;  // this warp's columns, in blocks of 16
-    const int quad = warp & 3, ch = (warp - 4) >> 2;
-    const int tq = lane & 3;
-    // rows ri = 4 h + 2 hb + r8: row block h, 16-lane half hb, lane t/4 + 8 r8;
-    // .x / .y accumulate the even / odd column of the thread's pairs
-    float2 acc[8][3];
+    constexpr int NU = NC / 16;  // units of 16 columns
+    const int quad = warp & 3, h = (warp - kFwdEpi0) >> 2;
+    const int tq = lane & 3, tr = lane >> 2;
+    // rows ri = hb * 2 + r8: 16-lane half hb, lane t/4 + 8 r8; .x / .y
+    // accumulate the even / odd column of the thread's pairs
+    float2 acc[4][3];
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
       for (int c = 0; c < 3; ++c) acc[r][c] = make_float2(0.f, 0.f);
-    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ch * CW);
-    // one chunk: units (block n, row block h) in the order n-major, the next
-    // unit loading while one is used
-    auto chunk = [&](int b, const float* wp, auto sc_tag, auto nh_tag) {
+    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(h * NC);
+    // One chunk.  The exponentials of a unit are issued together with the
+    // colour sums of the one before, so that MUFU and FMA work overlap inside
+    // a warp; the next unit loads meanwhile.
+    auto chunk = [&](int b, const float* wp, auto sc_tag) {
       constexpr bool SC = decltype(sc_tag)::value;
-      constexpr int NH = decltype(nh_tag)::value, NU = NB * NH;
       uint32_t v[2][2][8];
-      float4 w01[2];
-      float2 w2[2], sc[2];
+      float4 w01[2][2];
+      float2 w2[2][2], sc[2];
       auto load = [&](int u) {
 #pragma unroll
         for (int hb = 0; hb < 2; ++hb)
-          tmem_ld16x256_x2_nowait(lane_base + ((uint32_t)(hb * 16) << 16) +
-                                      (uint32_t)((2 * b + u % NH) * NC + (u / NH) * 16),
-                                  v[u & 1][hb]);
+          tmem_ld16x256_x2_nowait(
+              lane_base + ((uint32_t)(hb * 16) << 16) + (uint32_t)(2 * b * NC + u * 16), v[u & 1][hb]);
+      };
+      auto exps = [&](int u, int k, int hb) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float sv = __uint_as_float(v[u & 1][hb][4 * k + j]);
+          if (SC) sv *= (j & 1) ? sc[k].y : sc[k].x;
+          v[u & 1][hb][4 * k + j] = __float_as_uint(ex2_approx(sv));
+        }
+      };
+      auto sums = [&](int u, int k, int hb) {
+#pragma unroll
+        for (int r8 = 0; r8 < 2; ++r8) {
+          const float2 e = make_float2(__uint_as_float(v[u & 1][hb][4 * k + 2 * r8]),
+                                       __uint_as_float(v[u & 1][hb][4 * k + 2 * r8 + 1]));
+          const int ri = 2 * hb + r8;
+          acc[ri][0] = __ffma2_rn(make_float2(w01[u & 1][k].x, w01[u & 1][k].y), e, acc[ri][0]);
+          acc[ri][1] = __ffma2_rn(make_float2(w01[u & 1][k].z, w01[u & 1][k].w), e, acc[ri][1]);
+          acc[ri][2] = __ffma2_rn(w2[u & 1][k], e, acc[ri][2]);
+        }
       };
       load(0);
 #pragma unroll
       for (int u = 0; u < NU; ++u) {
-        const int n = u / NH, h = u % NH;
-        if (h == 0) {
 #pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            const float* wk = wp + (8 * n + 4 * k) * 8;
-            w01[k] = *reinterpret_cast<const float4*>(wk);
-            w2[k] = *reinterpret_cast<const float2*>(wk + 4);
-            if (SC) sc[k] = *reinterpret_cast<const float2*>(wk + 6);
-          }
+        for (int k = 0; k < 2; ++k) {
+          const float* wk = wp + (8 * u + 4 * k) * 8;
+          w01[u & 1][k] = *reinterpret_cast<const float4*>(wk);
+          w2[u & 1][k] = *reinterpret_cast<const float2*>(wk + 4);
+          if (SC) sc[k] = *reinterpret_cast<const float2*>(wk + 6);
         }
-        uint32_t(&vu)[2][8] = v[u & 1];
         tmem_wait_ld();
-        tmem_reg_fence8(vu[0]);
-        tmem_reg_fence8(vu[1]);
-        if (u + 1 < NU) {
-          load(u + 1);
-        } else {
+        tmem_reg_fence8(v[u & 1][0]);
+        tmem_reg_fence8(v[u & 1][1]);
+        if (u == NU - 1) {
           // this warp's reads of buffer b are complete
           fence_before_sync();
-          warp_arrive(&acc_empty[b]);
+          warp_arrive(&acc_empty[2 * b + h]);
         }
-        // the unit's 16 exponentials first, in place (independent MUFU
-        // operations whose latency overlaps), then the colour sums
 #pragma unroll
         for (int k = 0; k < 2; ++k)
 #pragma unroll
-          for (int hb = 0; hb < 2; ++hb)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              float sv = __uint_as_float(vu[hb][4 * k + j]);
-              if (SC) sv *= (j & 1) ? sc[k].y : sc[k].x;
-              vu[hb][4 * k + j] = __float_as_uint(ex2_approx(sv));
-            }
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-          for (int hb = 0; hb < 2; ++hb)
-#pragma unroll
-            for (int r8 = 0; r8 < 2; ++r8) {
-              const float2 e = make_float2(__uint_as_float(vu[hb][4 * k + 2 * r8]),
-                                           __uint_as_float(vu[hb][4 * k + 2 * r8 + 1]));
-              const int ri = 4 * h + 2 * hb + r8;
-              acc[ri][0] = __ffma2_rn(make_float2(w01[k].x, w01[k].y), e, acc[ri][0]);
-              acc[ri][1] = __ffma2_rn(make_float2(w01[k].z, w01[k].w), e, acc[ri][1]);
-              acc[ri][2] = __ffma2_rn(w2[k], e, acc[ri][2]);
-            }
+          for (int hb = 0; hb < 2; ++hb) {
+            exps(u, k, hb);
+            if (u > 0) sums(u - 1, k, hb);
+          }
+        if (u + 1 < NU) load(u + 1);
       }
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int hb = 0; hb < 2; ++hb) sums(NU - 1, k, hb);
     };
-    for (int i = 0; i < nchunks; ++i) {
+    for (int i = 0; h < nh && i < nchunks; ++i) {
       const int s = i % CS, b = i & 1;
-      bool ok = warp_wait(&coef_full[s], (i / CS) & 1, abort_flag);
-      const int4 fl = *reinterpret_cast<const int4*>(&sflag[s][0]);
-      const bool scaled = (fl.x | fl.y | fl.z) != 0;
-      if (ok) ok = warp_wait(&acc_full[b], (i >> 1) & 1, abort_flag);
-      if (!ok) {
+      if (!warp_wait(&acc_full[2 * b + h], (i >> 1) & 1, abort_flag)) {
         if (lane == 0) fail();
         break;
       }
       fence_after_sync();
-      // weight pair entries of this thread: p = CW / 2 ch + 8 n + 4 k + tq
-      const float* wp = reinterpret_cast<const float*>(Cst + s * S::C_STAGE + 2 * S::B_BYTES) +
-                        (CW / 2 * ch + tq) * 8;
-      if (nh == 2) {
-        if (scaled) chunk(b, wp, BoolTag<true>{}, IntTag<2>{});
-        else chunk(b, wp, BoolTag<false>{}, IntTag<2>{});
-      } else {
-        if (scaled) chunk(b, wp, BoolTag<true>{}, IntTag<1>{});
-        else chunk(b, wp, BoolTag<false>{}, IntTag<1>{});
-      }
+      const int4 fl = *reinterpret_cast<const int4*>(&sflag[s][0]);
+      const bool scaled = (fl.x | fl.y | fl.z) != 0;
+      // weight pair entries of this thread: p = 8 u + 4 k + tq
+      const float* wp = reinterpret_cast<const float*>(Cst + s * S::C_STAGE + 2 * S::B_BYTES) + tq * 8;
+      if (scaled) chunk(b, wp, BoolTag<true>{});
+      else chunk(b, wp, BoolTag<false>{});
       warp_arrive(&coef_empty[s]);
     }
     // ---- row sums over the pair halves and the four threads sharing a lane
-    // (shuffles); thread tq keeps rows ri = tq and 4 + tq
+    // (shuffles); thread tq writes row ri = tq
+    if (h < nh && !*abort_flag) {
 #pragma unroll
-    for (int ri = 0; ri < 8; ++ri)
+      for (int ri = 0; ri < 4; ++ri) {
+        float rs[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        float v = acc[ri][c].x + acc[ri][c].y;
-        v += __shfl_xor_sync(0xffffffffu, v, 1);
-        v += __shfl_xor_sync(0xffffffffu, v, 2);
-        if ((ri & 3) == tq) rs[ri >> 2][c] = v;
+        for (int c = 0; c < 3; ++c) {
+          float v = acc[ri][c].x + acc[ri][c].y;
+          v += __shfl_xor_sync(0xffffffffu, v, 1);
+          v += __shfl_xor_sync(0xffffffffu, v, 2);
+          rs[c] = v;
+        }
+        const int qr = h * 128 + quad * 32 + (ri >> 1) * 16 + (ri & 1) * 8 + tr;
+        if (ri == tq && qr < nq) {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) a.y[(qt + qr) * 3 + c] = rs[c];
+        }
       }
-    // the second column half hands its sums over through the operand rows of
-    // stage 0 (every MMA that read them is complete: this warp saw the last
-    // chunk's acc_full, and no builder writes after it)
-    if (ch == 1 && !*abort_flag) {
-      float* dst = reinterpret_cast<float*>(Cst) + my_row * 3;
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) dst[h * 128 * 3 + c] = rs[h][c];
     }
   }
+  // A barrier counts a warp each time a part of it arrives: the issuer's lane
+  // and the other 31 come back together.
+  __syncwarp();
   fence_before_sync();
   __syncthreads();
-  if (warp >= 4 && warp < 8 && !*abort_flag) {
-    const float* o = reinterpret_cast<const float*>(Cst) + my_row * 3;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (h * 128 + my_row < nq) {
-        const long long q = qt + h * 128 + my_row;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) a.y[q * 3 + c] = nchunks > 0 ? rs[h][c] + o[h * 128 * 3 + c] : 0.0f;
-      }
-  }
-  if (warp == 12 && lane == 0) {
+  if (warp == kFwdIssuer && elect_one()) {
     // every MMA this thread issued has completed once this commit arrives
     mma_commit(&drain);
     if (!mbar_wait_bounded(&drain, 0, kWaitLimit)) fail();
   }
+  __syncwarp();
   fence_before_sync();
+  __syncthreads();
+  // a barrier must be invalidated before the next tile initialises it again
+  // (without, the second tile of a CTA saw phases of the first)
+  if (tid == 0)
+    for (int i = 0; i < FwdHSync::kBarriers; ++i) mbar_inval(&sy.coef_full[0] + i);
   __syncthreads();
 }
 
