@@ -12,13 +12,13 @@
 //                 [m_r - k_g sigma_r, m_r + k_g sigma_r] for every projection
 //                 (bytes), plus its first-projection bin blo * B + bhi
 //   radix sort    Gaussians by bin (stable, so ascending index inside a bin)
-//   cull_tile     one CTA per tile visits exactly the Gaussians whose first
-//                 projection range meets the tile's: bins (b, >= tlo) for
-//                 b <= thi are contiguous runs of the sorted order; the other
+//   cull_count    one CTA per group of tiles visits the Gaussians whose first
+//                 projection range meets the group's: bins (b, >= tlo) for
+//                 b <= thi are contiguous runs of the sorted order; all
 //                 projections are tested four at a time with byte-SIMD
-//                 compares; survivors are compacted with warp ballots and a
-//                 block prefix.  Run twice: count, then (after a scan of the
-//                 counts) fill.
+//                 compares, and the survivors' warp ballots stored per tile
+//   cull_fill     after a scan of the counts, one CTA per tile writes its
+//                 survivors from the ballots
 #include "common.cuh"
 #include "internal.h"
 #include "kernels.h"
@@ -240,7 +240,7 @@ __device__ bool condition_gaussian(const double* L, const double* m, const float
 }
 
 template <int N>
-__global__ void __launch_bounds__(128) prep_kernel(PrepArgs a) {
+__global__ void __launch_bounds__(32) prep_kernel(PrepArgs a) {
   constexpr int P = tri(N);
   constexpr int R = rec_floats(N);
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -441,116 +441,175 @@ __device__ __forceinline__ bool keys_overlap(const uint32_t* glo, const uint32_t
   return ok == 0xffffffffu;
 }
 
-// One CTA of CT_WARPS warps per tile.  The tile's sources (Gaussians whose
-// first-projection bucket range meets the tile's) are thi0 + 1 runs of the
-// bin-sorted order; warp w takes the contiguous slice w of their
-// concatenation (slice bounds at multiples of 32), walks it 32 elements at
-// a time (each lane tracks its run).  The count pass tests the remaining
-// projections, counts the survivors and stores the ballot of every 32
-// sources in masks[t][i / 32]; the fill pass reads the ballots back (no
-// key loads) and writes the survivors in order at the scanned offset of
-// (tile, warp), so the list order is the concatenation order.
+// Sources of a group of `group` consecutive tiles: the Gaussians whose
+// first-projection bucket range meets that of any of the tiles, thi0 + 1 runs
+// of the bin-sorted order (thi0 / tlo0: the group's largest / smallest first
+// bucket).  Every key test includes the first projection, so a tile's list
+// does not depend on the group, and neither does its order: ascending
+// positions of the bin-sorted order.  A slice of the runs' concatenation
+// (bounds at multiples of 32) belongs to each of the CTA's 8 warps.
+struct CullRuns {
+  long long rbeg[256], rpre[257], ws[8];
+};
 template <int KP>
-__global__ void __launch_bounds__(256) cull_tile_kernel(CullTileArgs a) {
-  constexpr int W = KP / 4;  // 32-bit words per key half (KP >= 8)
-  __shared__ long long rbeg[256];
-  __shared__ long long rpre[257];
-  __shared__ long long s_total;
-  __shared__ long long ws_[8];
-  const long long t = blockIdx.x;
+__device__ __forceinline__ int group_runs(const CullTileArgs& a, long long t0, CullRuns& s) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t tlo[W > 0 ? W : 1], thi[W > 0 ? W : 1];
   int tlo0 = 0, thi0 = 0;
   if (KP > 0) {
-    const uint32_t* tk = reinterpret_cast<const uint32_t*>(a.tkey + t * 2 * KP);
-#pragma unroll
-    for (int w = 0; w < W; ++w) { tlo[w] = tk[w]; thi[w] = tk[W + w]; }
-    tlo0 = a.tkey[t * 2 * KP];
-    thi0 = a.tkey[t * 2 * KP + KP];
+    tlo0 = 255;
+    for (int q = 0; q < a.group && t0 + q < a.T; ++q) {
+      const int l = a.tkey[(t0 + q) * 2 * KP], h = a.tkey[(t0 + q) * 2 * KP + KP];
+      tlo0 = l < tlo0 ? l : tlo0;
+      thi0 = h > thi0 ? h : thi0;
+    }
   }
   const int nb = KP > 0 ? a.B : 1;
   const int nr = thi0 + 1;  // first-projection bucket rows b = 0 .. thi0
-  {
-    long long len = 0;
-    if (tid < nr) {
-      long long b0 = a.binoff[(long long)tid * nb + tlo0];
-      long long b1 = a.binoff[(long long)(tid + 1) * nb];
-      rbeg[tid] = b0;
-      len = b1 > b0 ? b1 - b0 : 0;
-    }
-    long long v = tid < nr ? len : 0, incl = v;
+  long long len = 0;
+  if (tid < nr) {
+    long long b0 = a.binoff[(long long)tid * nb + tlo0];
+    long long b1 = a.binoff[(long long)(tid + 1) * nb];
+    s.rbeg[tid] = b0;
+    len = b1 > b0 ? b1 - b0 : 0;
+  }
+  long long incl = len;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      long long u = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += u;
-    }
-    if (lane == 31) ws_[warp] = incl;
-    __syncthreads();
-    long long off = 0;
-    for (int w = 0; w < warp; ++w) off += ws_[w];
-    if (tid < nr) rpre[tid] = incl - v + off;
-    if (tid == 255) rpre[nr] = incl + off;  // total (threads past nr add 0)
-    __syncthreads();
-    if (tid == 0) s_total = rpre[nr];
-    __syncthreads();
+  for (int o = 1; o < 32; o <<= 1) {
+    long long u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
   }
-  const long long n_src = s_total;
-  auto bound = [&](int w) -> long long {
-    const long long v = (n_src * w / 8 + 31) / 32 * 32;
-    return v < n_src ? v : n_src;
-  };
-  const long long lo = bound(warp), hi = warp == 7 ? n_src : bound(warp + 1);
-  uint32_t* masks = a.masks + t * a.mask_words;
-  // run of the slice's first element: largest r with rpre[r] <= lo
-  int r = 0;
-  {
-    int a0 = 0, b0 = nr - 1;
-    while (a0 < b0) {
-      int mid = (a0 + b0 + 1) >> 1;
-      if (rpre[mid] <= lo) a0 = mid; else b0 = mid - 1;
-    }
-    r = a0;
+  if (lane == 31) s.ws[warp] = incl;
+  __syncthreads();
+  long long off = 0;
+  for (int w = 0; w < warp; ++w) off += s.ws[w];
+  if (tid < nr) s.rpre[tid] = incl - len + off;
+  if (tid == 255) s.rpre[nr] = incl + off;  // total (threads past nr add 0)
+  __syncthreads();
+  return nr;
+}
+// run of source lo: the largest r with rpre[r] <= lo
+__device__ __forceinline__ int run_of(const CullRuns& s, int nr, long long lo) {
+  int a0 = 0, b0 = nr - 1;
+  while (a0 < b0) {
+    const int mid = (a0 + b0 + 1) >> 1;
+    if (s.rpre[mid] <= lo) a0 = mid; else b0 = mid - 1;
   }
-  const bool fill = a.ids != nullptr;
-  long long written = fill ? a.excl[t * 8 + warp] : 0;
-  long long count = 0;
+  return a0;
+}
+__device__ __forceinline__ long long slice_bound(long long n_src, int w) {
+  const long long v = (n_src * w / 8 + 31) / 32 * 32;
+  return w == 8 || v > n_src ? n_src : v;
+}
+
+// Count pass: one CTA per group of TG tiles.  A warp reads 32 key rows once
+// and tests them against every tile of the group, counts the survivors and
+// stores the ballot of every 32 sources in masks[t][i / 32].  Bound by the
+// tests' instructions: up to 128 buckets (SMALL) every byte is below 128, and
+// with bit 7 set in the minuends a <= b in all four bytes of a word is one
+// subtraction (no byte borrows) whose bits 7 stay; the general byte compares
+// take several instructions each.
+template <int KP, int TG, bool SMALL>
+__global__ void __launch_bounds__(256) cull_count_kernel(CullTileArgs a) {
+  constexpr int W = KP / 4;  // 32-bit words per key half (KP >= 8)
+  __shared__ CullRuns s;
+  const long long t0 = (long long)blockIdx.x * TG;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t tlo[TG][W > 0 ? W : 1], thi[TG][W > 0 ? W : 1];
+#pragma unroll
+  for (int q = 0; q < TG; ++q) {
+    const long long t = t0 + q < a.T ? t0 + q : a.T - 1;
+    const uint32_t* tk = reinterpret_cast<const uint32_t*>(a.tkey + t * 2 * KP);
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      tlo[q][w] = tk[w];
+      thi[q][w] = SMALL ? tk[W + w] | 0x80808080u : tk[W + w];
+    }
+  }
+  const int nr = group_runs<KP>(a, t0, s);
+  const long long n_src = s.rpre[nr];
+  const long long lo = slice_bound(n_src, warp), hi = slice_bound(n_src, warp + 1);
+  int r = run_of(s, nr, lo);
+  long long count[TG];
+#pragma unroll
+  for (int q = 0; q < TG; ++q) count[q] = 0;
   for (long long i0 = lo; i0 < hi; i0 += 32) {
     const long long i = i0 + lane;
-    unsigned bal;
-    if (!fill) {
-      bool pass = false;
-      if (i < hi) {
-        if (KP > 0) {
-          while (r + 1 < nr && rpre[r + 1] <= i) ++r;
-          const long long pos = rbeg[r] + (i - rpre[r]);
-          // keys in bin-sorted order: a warp reads consecutive rows, 16 bytes
-          // per load (rows are 2 KP = 16, 32, 48 or 64 bytes, 16-byte aligned)
-          const uint4* gk = reinterpret_cast<const uint4*>(a.gkey + (size_t)pos * 2 * KP);
-          uint32_t row[2 * W > 4 ? 2 * W : 4];
+    uint32_t row[2 * W > 4 ? 2 * W : 4];
+    const bool in = i < hi;
+    if (KP > 0 && in) {
+      while (r + 1 < nr && s.rpre[r + 1] <= i) ++r;
+      const long long pos = s.rbeg[r] + (i - s.rpre[r]);
+      // keys in bin-sorted order: a warp reads consecutive rows, 16 bytes
+      // per load (rows are 2 KP = 16, 32, 48 or 64 bytes, 16-byte aligned)
+      const uint4* gk = reinterpret_cast<const uint4*>(a.gkey + (size_t)pos * 2 * KP);
 #pragma unroll
-          for (int v = 0; v < (2 * W) / 4; ++v) {
-            const uint4 q = __ldg(gk + v);
-            row[4 * v] = q.x; row[4 * v + 1] = q.y; row[4 * v + 2] = q.z; row[4 * v + 3] = q.w;
-          }
-          pass = keys_overlap(row, row + W, tlo, thi, W);
-        } else {
-          pass = true;
-        }
+      for (int v = 0; v < (2 * W) / 4; ++v) {
+        const uint4 x = __ldg(gk + v);
+        row[4 * v] = x.x; row[4 * v + 1] = x.y; row[4 * v + 2] = x.z; row[4 * v + 3] = x.w;
       }
-      bal = __ballot_sync(0xffffffffu, pass);
-      if (lane == 0) masks[i0 >> 5] = bal;
-    } else {
-      bal = masks[i0 >> 5];
-      if ((bal >> lane) & 1u) {
-        while (r + 1 < nr && rpre[r + 1] <= i) ++r;
-        const long long src = rbeg[r] + (i - rpre[r]);
-        const long long pos = written + count + __popc(bal & ((1u << lane) - 1u));
-        if (pos < a.E_cap) a.ids[pos] = a.sorted_ids[src];
+      if (SMALL) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) row[W + w] |= 0x80808080u;
       }
     }
-    count += __popc(bal);
+#pragma unroll
+    for (int q = 0; q < TG; ++q) {
+      bool pass = in;
+      if (KP > 0 && SMALL) {
+        uint32_t ok = 0x80808080u;
+#pragma unroll
+        for (int w = 0; w < W; ++w) ok &= (thi[q][w] - row[w]) & (row[W + w] - tlo[q][w]);
+        pass = in && ok == 0x80808080u;
+      } else if (KP > 0) {
+        pass = in && keys_overlap(row, row + W, tlo[q], thi[q], W);
+      }
+      const unsigned bal = __ballot_sync(0xffffffffu, pass);
+      if (lane == 0 && t0 + q < a.T) a.masks[(t0 + q) * a.mask_words + (i0 >> 5)] = bal;
+      count[q] += __popc(bal);
+    }
   }
-  if (!fill && lane == 0) a.counts[t * 8 + warp] = count;
+#pragma unroll
+  for (int q = 0; q < TG; ++q)
+    if (lane == 0 && t0 + q < a.T) a.counts[(t0 + q) * 8 + warp] = count[q];
+}
+
+// Fill pass: one CTA per tile reads its ballots back (no key loads) and
+// writes the survivors in order at the scanned offset of (tile, warp).
+template <int KP>
+__global__ void __launch_bounds__(256) cull_fill_kernel(CullTileArgs a) {
+  __shared__ CullRuns s;
+  const long long t = blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nr = group_runs<KP>(a, t / a.group * a.group, s);
+  const long long n_src = s.rpre[nr];
+  const long long lo = slice_bound(n_src, warp), hi = slice_bound(n_src, warp + 1);
+  int r = run_of(s, nr, lo);
+  const uint32_t* masks = a.masks + t * a.mask_words;
+  long long written = a.excl[t * 8 + warp];
+  // four ballots, then their survivors' ids, in flight at a time
+  constexpr int U = 4;
+  for (long long i0 = lo; i0 < hi; i0 += 32 * U) {
+    unsigned bal[U];
+    int id[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) bal[u] = i0 + 32 * u < hi ? masks[(i0 >> 5) + u] : 0u;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if ((bal[u] >> lane) & 1u) {
+        const long long i = i0 + 32 * u + lane;
+        while (r + 1 < nr && s.rpre[r + 1] <= i) ++r;
+        id[u] = __ldg(a.sorted_ids + s.rbeg[r] + (i - s.rpre[r]));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if ((bal[u] >> lane) & 1u) {
+        const long long pos = written + __popc(bal[u] & ((1u << lane) - 1u));
+        if (pos < a.E_cap) a.ids[pos] = id[u];
+      }
+      written += __popc(bal[u]);
+    }
+  }
 }
 
 // Key rows in bin-sorted order: dst[p] = src[sorted[p]] (2 KP bytes a row).
@@ -601,8 +660,11 @@ int launch_tile_keys(const float* tb, long long T, int k, int KP, int B, const f
 
 int launch_prep(int N, const PrepArgs& a, cudaStream_t s) {
   if (a.Ge <= 0) return 0;
-  unsigned blocks = (unsigned)ceil_div(a.Ge, 128);
-#define L_PREP(n) prep_kernel<n><<<blocks, 128, 0, s>>>(a)
+  // one warp per block: the kernel is bound by FP64 arithmetic, a few lanes of
+  // it per SM, so that a few thousand Gaussians have to spread over every SM
+  // (5,000 at N = 8 are 40 blocks of 128)
+  unsigned blocks = (unsigned)ceil_div(a.Ge, 32);
+#define L_PREP(n) prep_kernel<n><<<blocks, 32, 0, s>>>(a)
   NDG_SWITCH_N(N, L_PREP)
 #undef L_PREP
   return 1;
@@ -617,16 +679,39 @@ int launch_permute_keys(const uint8_t* src, const int32_t* sorted, int n, int KP
   return 1;
 }
 
-int launch_cull_tile(int KP, const CullTileArgs& a, long long T, cudaStream_t s) {
+// Tiles per CTA of the count pass: four while that still gives every SM four
+// CTAs (a key row is then read once for four tiles), fewer for few tiles.
+int cull_group(int KP, long long T) {
+  if (KP == 0) return 1;
+  return T >= 4 * 4 * 152 ? 4 : T >= 2 * 4 * 152 ? 2 : 1;
+}
+
+int launch_cull_tile(int KP, const CullTileArgs& args, long long T, cudaStream_t s) {
   if (T <= 0) return 0;
+  CullTileArgs a = args;
+  a.T = T;
+  a.group = cull_group(KP, T);
+  const unsigned groups = (unsigned)ceil_div<long long>(T, a.group);
+  const bool small = a.B <= 128;
+#define L_CC(K, TG)                                                          \
+  if (small) cull_count_kernel<K, TG, true><<<groups, 256, 0, s>>>(a);       \
+  else cull_count_kernel<K, TG, false><<<groups, 256, 0, s>>>(a);
+#define L_CT(K)                                                              \
+  if (a.ids) cull_fill_kernel<K><<<(unsigned)T, 256, 0, s>>>(a);             \
+  else if (a.group == 4) { L_CC(K, 4) }                                      \
+  else if (a.group == 2) { L_CC(K, 2) }                                      \
+  else { L_CC(K, 1) }                                                        \
+  break;
   switch (KP) {
-    case 0: cull_tile_kernel<0><<<(unsigned)T, 256, 0, s>>>(a); break;
-    case 8: cull_tile_kernel<8><<<(unsigned)T, 256, 0, s>>>(a); break;
-    case 16: cull_tile_kernel<16><<<(unsigned)T, 256, 0, s>>>(a); break;
-    case 24: cull_tile_kernel<24><<<(unsigned)T, 256, 0, s>>>(a); break;
-    case 32: cull_tile_kernel<32><<<(unsigned)T, 256, 0, s>>>(a); break;
+    case 0: L_CT(0)
+    case 8: L_CT(8)
+    case 16: L_CT(16)
+    case 24: L_CT(24)
+    case 32: L_CT(32)
     default: return 0;
   }
+#undef L_CT
+#undef L_CC
   return 1;
 }
 

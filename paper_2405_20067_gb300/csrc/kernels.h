@@ -40,6 +40,8 @@ struct CullTileArgs {
   long long E_cap;
   uint32_t* masks;            // [T][mask_words] survivor ballots of the count pass
   long long mask_words;       // per tile: >= ceil(max sources / 32) + 8
+  long long T;                // set by launch_cull_tile: tiles, and tiles per
+  int group;                  // CTA of the count pass
 };
 
 struct FwdArgs {
