@@ -35,7 +35,7 @@
 //
 // CTA = one tile of up to 256 queries, 416 threads, one CTA per SM:
 //   warps 0-3   builders: coefficient rows of chunk i into coefficient stage
-//               i % CS, the chunk's per-candidate data (m~, w / rho, entry,
+//               i % CS (N = 10, 11: into tensor memory, one stage), the chunk's per-candidate data (m~, w / rho, entry,
 //               row factor, rho) into stash slot i % SS;
 //   warp 12     MMA issuer (one lane): MMA 1 of unit u + LEAD, then MMA 2 of u;
 //   warps 4-11  epilogue: warp w owns TMEM lanes 32 (w % 4) .. + 31 (its
@@ -43,7 +43,7 @@
 //               last unit of chunk i it forms half of the record parts of
 //               chunk i - 1 (the builders held the next chunk's records in
 //               registers, and the chain there spilled).
-// TMEM: NBUF S buffers of 128 columns, then two D buffers.  Every wait is
+// TMEM: NBUF S buffers of 128 columns, two D buffers, the coefficient rows.  Every wait is
 // bounded; a timeout records NDG_ERR_TIMEOUT and the CTA lets its issued
 // MMAs finish (bounded) before it frees tensor memory.
 #include <cuda_fp16.h>
@@ -85,7 +85,17 @@ struct BwdBShape {
   static constexpr uint32_t PHI_BYTES = 32u * GRP;       // 256 queries
   static constexpr uint32_t SBO_C = (KP / 8) * 128;      // coefficient rows: 8-row groups
   static constexpr uint32_t C_BYTES = (uint32_t)NC * KP * 2;
-  static constexpr uint32_t C_STAGE = 2 * C_BYTES;       // hi, lo
+  // The coefficient rows are MMA 1's A operand in tensor memory where a stage
+  // of them fits beside S and D and their share of the shared-memory pipe is
+  // large: with them there an MMA reads 8 KB of operands from it for 128
+  // columns, the whole pipe's rate.  Measured: N = 10 fit 35.1 -> 30.1 ms,
+  // N = 11 evaluation (10,000 Gaussians, 32,768 queries) 561 -> 477 us; N = 7
+  // 767 -> 755 us and N = 8 2,178 -> 2,229 us (20,000 + children, 65,536
+  // queries), where three stages ahead are worth as much, so those keep
+  // shared memory.  N = 9 and 12 have no room.
+  static constexpr uint32_t TM_C = TM_D + 2 * ND;
+  static constexpr bool CTM = KP > 48 && TM_C + KP <= 512;
+  static constexpr uint32_t C_STAGE = CTM ? 0 : 2 * C_BYTES;  // hi, lo
   // stash slot: SV fields per candidate, field-major ([SV][NC]: lane j
   // reads word j of a field, conflict-free): m~ (N), w / rho (3), entry,
   // row factor, rho; then the two column halves' sum_q e dy' (float4 each)
@@ -96,7 +106,8 @@ struct BwdBShape {
   static constexpr uint32_t OUT_BYTES = 16u * PQS * 16;
   static constexpr uint32_t FIXED = PHI_BYTES + SS * SLOT + DYC + 8 * OUT_BYTES + 128 + 4096;
   // coefficient stages: as many as fit (up to 3; N = 12 has room for one)
-  static constexpr int CS = FIXED + 3 * C_STAGE <= 227u * 1024u   ? 3
+  static constexpr int CS = CTM ? 1
+                            : FIXED + 3 * C_STAGE <= 227u * 1024u   ? 3
                             : FIXED + 2 * C_STAGE <= 227u * 1024u ? 2
                                                                   : 1;
   static constexpr uint32_t SMEM_USED = FIXED - 4096 + CS * C_STAGE;
@@ -324,7 +335,7 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
     };
     auto build = [&](int i, const float4 (&cur)[R4], int slot) -> bool {
       const int s = i % CS;
-      if (i >= CS && !warp_wait(&coef_empty[s], ((i / CS) - 1) & 1, abort_flag)) return false;
+      if (!S::CTM && i >= CS && !warp_wait(&coef_empty[s], ((i / CS) - 1) & 1, abort_flag)) return false;
       if (i >= SS && !warp_wait(&stash_empty[i % SS], ((i / SS) - 1) & 1, abort_flag)) return false;
       float buf[S::R];
 #pragma unroll
@@ -365,7 +376,13 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
 #pragma unroll
         for (int k = 0; k < KP; ++k) coef[k] *= down;
       }
+      // one stage in tensor memory: MMA 1 of the chunk before has read it
+      if (S::CTM && i >= 1) {
+        if (!warp_wait(&coef_empty[0], (i - 1) & 1, abort_flag)) return false;
+        fence_after_sync();
+      }
       uint8_t* st = Cst + s * S::C_STAGE;
+      const uint32_t tc = tmem + ((uint32_t)(warp * 32) << 16) + S::TM_C;
 #pragma unroll
       for (int k = 0; k < KP; k += 8) {
         uint4 h, l;
@@ -373,11 +390,21 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
         split_hb(coef[k + 2], coef[k + 3], h.y, l.y);
         split_hb(coef[k + 4], coef[k + 5], h.z, l.z);
         split_hb(coef[k + 6], coef[k + 7], h.w, l.w);
-        const uint32_t off = coff(j, k, S::SBO_C);
-        *reinterpret_cast<uint4*>(st + off) = h;
-        *reinterpret_cast<uint4*>(st + S::C_BYTES + off) = l;
+        if constexpr (S::CTM) {
+          tmem_st4(tc + (uint32_t)(k / 2), h);
+          tmem_st4(tc + (uint32_t)(KP / 2 + k / 2), l);
+        } else {
+          const uint32_t off = coff(j, k, S::SBO_C);
+          *reinterpret_cast<uint4*>(st + off) = h;
+          *reinterpret_cast<uint4*>(st + S::C_BYTES + off) = l;
+        }
       }
-      fence_proxy_async();
+      if constexpr (S::CTM) {
+        tmem_wait_st();
+        fence_before_sync();
+      } else {
+        fence_proxy_async();
+      }
       warp_arrive(&coef_full[s]);
       // stash: m~, w / rho, entry, row factor, rho (read by the epilogue and
       // the chain).  rho, a power of two, brings the largest weight into
@@ -453,9 +480,16 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
 #pragma unroll
         for (int ks = 0; ks < KP / 16; ++ks) {
           const uint64_t ko = (uint64_t)ks * 16u;  // two 128-byte cores per K step
-          mma_f16(d, dch + ko, dph + ko, IDESC1, ks > 0 ? 1u : 0u);
-          mma_f16(d, dch + ko, dph + PHI_LO + ko, IDESC1, 1u);
-          mma_f16(d, dch + C_LO + ko, dph + ko, IDESC1, 1u);
+          if constexpr (S::CTM) {
+            const uint32_t ch = tmem + S::TM_C + 8u * ks;
+            mma_f16_ts(d, ch, dph + ko, IDESC1, ks > 0 ? 1u : 0u);
+            mma_f16_ts(d, ch, dph + PHI_LO + ko, IDESC1, 1u);
+            mma_f16_ts(d, ch + KP / 2, dph + ko, IDESC1, 1u);
+          } else {
+            mma_f16(d, dch + ko, dph + ko, IDESC1, ks > 0 ? 1u : 0u);
+            mma_f16(d, dch + ko, dph + PHI_LO + ko, IDESC1, 1u);
+            mma_f16(d, dch + C_LO + ko, dph + ko, IDESC1, 1u);
+          }
         }
         mma_commit(&s_full[sb]);
         if (h == nh - 1) mma_commit(&coef_empty[s]);

@@ -25,7 +25,7 @@
 //     per 128 bytes), the weight loads and the coefficient rows, was 68%
 //     (N = 6) to 82% (N = 10) busy with Phi as a shared-memory operand.  Phi,
 //     the same for all of a tile's chunks, is the A operand in tensor memory
-//     (hi and lo; N >= 10 has room for hi only and keeps lo in shared memory),
+//     (hi and lo; N = 10, 11 keep one block's lo in shared memory, N = 12 both),
 //     and the chunks are of 96 candidates so that two double-buffered
 //     accumulators and Phi share the 512 columns (an MMA of 96 columns costs
 //     its share of one of 128);
@@ -37,7 +37,7 @@
 //     columns are issued with the sums of the 16 before.
 // Measured, kernel alone: N = 6 256 x 256 frame (10,000 Gaussians) 235 -> 178
 // us, N = 8 701 x 397 (60,000) 5.72 -> 4.20 ms, N = 10 480 x 272 (100,000)
-// 6.79 -> 5.62 ms, N = 10 1080p (500,000) 491 -> 410 ms, N = 12 evaluation
+// 6.79 -> 5.37 ms, N = 10 1080p (500,000) 491 -> 392 ms, N = 12 evaluation
 // (10,000, 32,768 queries) 303 -> 233 us.  Four builders with 13 warps and
 // eight rows per weight load measured 124 us where this takes 112 (N = 8,
 // 5,000 Gaussians; 159 at first).
@@ -100,11 +100,12 @@ struct FwdHShape {
   static constexpr uint32_t SBO = (KP / 8) * 128;  // 8-row group stride (bytes)
   // tensor memory: four accumulators (buffer, row block) of NC columns, then
   // Phi as the MMAs' A operand, KP / 2 columns per row block and half: hi of
-  // both blocks, and lo too where the 512 columns hold it (N <= 9)
+  // both blocks, and lo of as many (LO_TM) as the 512 columns hold: both for
+  // N <= 9, one for N = 10, 11
   static constexpr uint32_t TM_PHI = 4u * NC;
-  static constexpr bool LO_TM = TM_PHI + 2 * KP <= 512;
+  static constexpr int LO_TM = TM_PHI + 2 * KP <= 512 ? 2 : TM_PHI + KP + KP / 2 <= 512 ? 1 : 0;
   static_assert(TM_PHI + KP <= 512, "tensor memory");
-  static constexpr uint32_t PHI_BYTES = LO_TM ? 0 : 256u * KP * 2;  // lo half in shared memory
+  static constexpr uint32_t PHI_BYTES = (2 - LO_TM) * 128u * KP * 2;  // the other lo halves, in shared memory
   static constexpr uint32_t HALF_BYTES = 128u * KP * 2;  // one 128-row block of it
   static constexpr uint32_t B_BYTES = (uint32_t)NC * KP * 2;
   static constexpr uint32_t W_BYTES = (uint32_t)NC * 16;  // w0 w0' w1 w1' w2 w2' k k' per pair
@@ -258,8 +259,8 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t) {
       split_h2(phi[k + 4], phi[k + 5], h.z, l.z);
       split_h2(phi[k + 6], phi[k + 7], h.w, l.w);
       tmem_st4(ph + (uint32_t)(k / 2), h);
-      if constexpr (S::LO_TM) tmem_st4(ph + (uint32_t)(KP + k / 2), l);
-      else *reinterpret_cast<uint4*>(Alo + kmajor_off_h(row, k, S::SBO)) = l;
+      if (row < 128 * S::LO_TM) tmem_st4(ph + (uint32_t)(KP + k / 2), l);
+      else *reinterpret_cast<uint4*>(Alo + kmajor_off_h(row - 128 * S::LO_TM, k, S::SBO)) = l;
     }
     tmem_wait_st();
   }
@@ -495,13 +496,13 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t) {
           fence_after_sync();
           const uint32_t d = tmem + (uint32_t)((2 * b + h) * NC);
           const uint32_t ah = tmem + S::TM_PHI + (uint32_t)(h * (KP / 2));
-          const uint64_t dal = dA0 + (uint64_t)((h * S::HALF_BYTES) >> 4);
+          const uint64_t dal = dA0 + (uint64_t)(((h - S::LO_TM) * (int)S::HALF_BYTES) >> 4);
 #pragma unroll
           for (int ks = 0; ks < KP / 16; ++ks) {
             const uint64_t ko = (uint64_t)ks * 16u;  // two 16-byte core matrices per K step
             mma_f16_ts(d, ah + 8u * ks, dbh + ko, IDESC, ks > 0 ? 1u : 0u);
             mma_f16_ts(d, ah + 8u * ks, dbh + B_LO + ko, IDESC, 1u);
-            if constexpr (S::LO_TM) mma_f16_ts(d, ah + KP + 8u * ks, dbh + ko, IDESC, 1u);
+            if (h < S::LO_TM) mma_f16_ts(d, ah + KP + 8u * ks, dbh + ko, IDESC, 1u);
             else mma_f16(d, dal + ko, dbh + ko, IDESC, 1u);
           }
           mma_commit(&acc_full[2 * b + h]);
