@@ -30,7 +30,7 @@
 // [-1, 1], and coefficient rows above 2^14 are divided by a power of two that
 // the epilogue multiplies back before the exponential.
 //
-// CTA = one tile of up to 256 queries = up to two units of 128 queries,
+// CTA = one tile (or a part of its candidates) of up to 256 queries = up to two units of 128 queries,
 // 416 threads, one CTA per SM (all 512 TMEM columns):
 //   warps 0-3   builders: coefficient rows of a chunk of 128 candidates into
 //               one of CS stages (as in the forward), one arrival per warp;
@@ -175,6 +175,11 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long t = blockIdx.x;
+  {
+    long long b = a.offsets[t], e = a.offsets[t + 1];
+    part_range(b, e, NC);
+    if (b >= e) return;
+  }
   const long long qt = t * a.tile;
   const int nq = (int)(a.Q - qt < a.tile ? a.Q - qt : a.tile);
   const int nh = (nq + S::UQ - 1) / S::UQ;  // units (blocks of UQ queries) per chunk
@@ -281,7 +286,8 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = tmem_base;
-  const long long beg = a.offsets[t], end = a.offsets[t + 1];
+  long long beg = a.offsets[t], end = a.offsets[t + 1];
+  part_range(beg, end, NC);
   const int nchunks = (int)((end - beg + NC - 1) / NC);
   const int U = nchunks * nh;
   volatile int* abort_flag = &s_abort;
@@ -655,11 +661,12 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
 
 int launch_bwd_h(int N, const BwdArgs& a, long long T, cudaStream_t s) {
   if (T <= 0) return 0;
+  const dim3 grid((unsigned)T, (unsigned)split_parts(N, T, kSMs));  // one CTA per SM
 #define L_BH(n)                                                                         \
   {                                                                                     \
     cudaFuncSetAttribute(bwd_h_kernel<n>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
                          (int)BwdHShape<n>::SMEM);                                      \
-    bwd_h_kernel<n><<<(unsigned)T, 416, BwdHShape<n>::SMEM, s>>>(a);                    \
+    bwd_h_kernel<n><<<grid, 416, BwdHShape<n>::SMEM, s>>>(a);                    \
   }
   switch (N) {
     case 1: L_BH(1); break;

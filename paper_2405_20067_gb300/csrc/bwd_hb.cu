@@ -33,7 +33,7 @@
 // dl/dw] (dl/dM = 2 M sum G and dl/dm = 2 A sum v follow per Gaussian after
 // the segmented sum), written in entry order.
 //
-// CTA = one tile of up to 256 queries, 416 threads, one CTA per SM:
+// CTA = one tile (or a part of its candidates) of up to 256 queries, 416 threads, one CTA per SM:
 //   warps 0-3   builders: coefficient rows of chunk i into coefficient stage
 //               i % CS (N = 10, 11: into tensor memory, one stage), the chunk's per-candidate data (m~, w / rho, entry,
 //               row factor, rho) into stash slot i % SS;
@@ -190,6 +190,9 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long t = blockIdx.x;
+  long long beg = a.offsets[t], end = a.offsets[t + 1];
+  part_range(beg, end, NC);
+  if (beg >= end) return;
   const long long qt = t * a.tile;
   const int nq = (int)(a.Q - qt < a.tile ? a.Q - qt : a.tile);
   const int nh = (nq + S::UQ - 1) / S::UQ;  // units per chunk
@@ -300,7 +303,6 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = tmem_base;
-  const long long beg = a.offsets[t], end = a.offsets[t + 1];
   const int nchunks = (int)((end - beg + NC - 1) / NC);
   const int U = nchunks * nh;
   volatile int* abort_flag = &s_abort;
@@ -790,11 +792,12 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
 
 int launch_bwd_hb(int N, const BwdArgs& a, long long T, cudaStream_t s) {
   if (T <= 0) return 0;
+  const dim3 grid((unsigned)T, (unsigned)split_parts(N, T, kSMs));  // one CTA per SM
 #define L_BB(n)                                                                         \
   {                                                                                     \
     cudaFuncSetAttribute(bwd_hb_kernel<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                          (int)BwdBShape<n>::SMEM);                                      \
-    bwd_hb_kernel<n><<<(unsigned)T, 416, BwdBShape<n>::SMEM, s>>>(a);                   \
+    bwd_hb_kernel<n><<<grid, 416, BwdBShape<n>::SMEM, s>>>(a);                   \
   }
   switch (N) {
     case 1: L_BB(1); break;

@@ -54,6 +54,35 @@ __device__ __forceinline__ int clampi(int v, int a, int b) { return v < a ? a : 
 template <typename T>
 __host__ __device__ inline T ceil_div(T a, T b) { return (a + b - 1) / b; }
 
+// ---- several CTAs per tile in the backward -------------------------------------
+// An entry's record depends on its own Gaussian and the tile's queries alone,
+// so a tile's candidates may be split over CTAs (grid y) without changing a
+// bit.  Few tiles leave SMs idle and a last wave nearly empty; every part pays
+// the tile's setup again, taken as 1/25 of an average tile, and as 1/5 for
+// N < 6, whose tiles are cheap (N = 3, 512 tiles: two parts, which 1/25 would
+// choose, measured 119 us against 109 to 114 for one).  slots: CTAs resident on the chip.  Measured:
+// N = 6, 16 tiles 406 -> 42 us, N = 6 FP32, 64 tiles 128 -> 52 us and 1,024
+// tiles 5.20 -> 4.31 ms, N = 10, 63 tiles of 128 queries 318 -> 138 us (start
+// against now, other changes of the TC kernels included).
+constexpr int kSMs = 152;
+inline int split_parts(int N, long long T, int slots) {
+  int best = 1;
+  double cost = 1e30;
+  const double setup = N < 6 ? 0.2 : 0.04;
+  for (int S = 1; S <= 8; ++S) {
+    const double c = (double)ceil_div<long long>(T * S, slots) * (1.0 / S + setup);
+    if (c < cost) { cost = c; best = S; }
+  }
+  return best;
+}
+// The part blockIdx.y of gridDim.y of entries [beg, end), in steps of `step`.
+__device__ __forceinline__ void part_range(long long& beg, long long& end, int step) {
+  const long long n = (end - beg + step - 1) / step, p = blockIdx.y, S = gridDim.y;
+  const long long e = beg + n * (p + 1) / S * step;
+  beg += n * p / S * step;
+  end = e < end ? e : end;
+}
+
 // ---- tile centre ---------------------------------------------------------------
 // Midpoint of the tile's bounding box (per dimension), computed by the CTA:
 // the kernels evaluate z = M (x - c) - M (m - c), which keeps the products

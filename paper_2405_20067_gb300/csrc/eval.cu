@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(LOSS_BLOCKS) loss_final_kernel(const double* _
 }
 
 // ---- backward partials ------------------------------------------------------------
-// One CTA of 128 threads per tile; each thread owns two candidates (the two
+// One CTA of 128 threads per tile or part of its candidates; each thread owns two candidates (the two
 // lanes of packed FP32x2 instructions) and loops over the tile's queries,
 // read from shared memory as (x - c, dy) duplicated into both lanes.  With
 // z' = kappa z: beta = e sum_c dy_c w_c, and the partial record of an entry
@@ -224,6 +224,9 @@ __global__ void __launch_bounds__(128) bwd_kernel(BwdArgs a) {
   __shared__ float sctr[N];
   const long long t = blockIdx.x;
   const int tid = threadIdx.x;
+  long long beg = a.offsets[t], end = a.offsets[t + 1];
+  part_range(beg, end, 256);
+  if (beg >= end) return;
   const long long q0 = t * a.tile;
   const int nq = (int)(a.Q - q0 < a.tile ? a.Q - q0 : a.tile);
   {
@@ -254,7 +257,6 @@ __global__ void __launch_bounds__(128) bwd_kernel(BwdArgs a) {
     }
   }
   __syncthreads();
-  const long long beg = a.offsets[t], end = a.offsets[t + 1];
   for (long long c0 = beg; c0 < end; c0 += 256) {
     const long long cid[2] = {c0 + tid, c0 + 128 + tid};
     float2 M2[P], b2[N], w2[3];
@@ -702,7 +704,9 @@ int launch_loss(const float* y, const float* target, float* dy, long long n, dou
 
 int launch_bwd(int N, const BwdArgs& a, long long T, cudaStream_t s) {
   if (T <= 0) return 0;
-#define L_BWD(n) bwd_kernel<n><<<(unsigned)T, 128, 0, s>>>(a)
+  // three resident CTAs of 128 threads per SM
+  const dim3 grid((unsigned)T, (unsigned)split_parts(N, T, 3 * kSMs));
+#define L_BWD(n) bwd_kernel<n><<<grid, 128, 0, s>>>(a)
   NDG_SWITCH_N(N, L_BWD)
 #undef L_BWD
   return 1;

@@ -37,7 +37,7 @@
 //     columns are issued with the sums of the 16 before.
 // Measured, kernel alone: N = 6 256 x 256 frame (10,000 Gaussians) 235 -> 178
 // us, N = 8 701 x 397 (60,000) 5.72 -> 4.20 ms, N = 10 480 x 272 (100,000)
-// 6.79 -> 5.37 ms, N = 10 1080p (500,000) 491 -> 392 ms, N = 12 evaluation
+// 6.79 -> 5.37 ms, N = 10 1080p (500,000) 491 -> 397 ms, N = 12 evaluation
 // (10,000, 32,768 queries) 303 -> 233 us.  Four builders with 13 warps and
 // eight rows per weight load measured 124 us where this takes 112 (N = 8,
 // 5,000 Gaussians; 159 at first).
