@@ -19,8 +19,8 @@
 // CTA = one tile of up to 256 queries (two M = 128 row blocks sharing the
 // candidate operand), 544 threads (96 registers), one CTA per SM.  What bounds
 // the tile: at N = 6 the epilogue's chain of exponentials and colour sums, at
-// N = 10 the builders and the MMAs (30 of 48 cycles per chunk).  What the
-// layout answers to:
+// N = 10 the MMAs (30 per chunk, at 70 cycles each against 48 alone, behind
+// the shared-memory pipe).  What the layout answers to:
 //   * the shared-memory pipe, shared by the MMAs' operand reads (a wavefront
 //     per 128 bytes), the weight loads and the coefficient rows, was 68%
 //     (N = 6) to 82% (N = 10) busy with Phi as a shared-memory operand.  Phi,
@@ -312,9 +312,9 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t) {
       bool ok = true;
       cp_async_wait_all();
       __syncwarp();
-      // N >= 9: the record stays in its row and is read twice (112 to 200 of
-      // a thread's 96 registers' worth would be spilled otherwise); smaller
-      // ones are read into registers and the next group's copies start at once.
+      // N >= 9: the record stays in its row and is read twice (in registers it
+      // spilled, N = 12 evaluation 551 us against 233); smaller ones are read
+      // into registers and the next group's copies start at once.
       constexpr bool STREAM = N >= 9;
       float4* mine = rows + lane * S::REC_STRIDE;
       if (g_cur < 0) {

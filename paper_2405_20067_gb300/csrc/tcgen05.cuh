@@ -69,22 +69,9 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// 16x256b.x4 load without the wait: 16 lanes x 32 columns.  Thread t gets,
+// 16x256b.x2 load without the wait: 16 lanes x 16 columns.  Thread t gets,
 // for each 8-column group k, registers 4k, 4k+1 = lane t/4, columns
 // 8k + 2 (t % 4) + {0, 1}, and 4k+2, 4k+3 = lane t/4 + 8, same columns.
-__device__ __forceinline__ void tmem_ld16x256_x4_nowait(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
-      "%12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-
-// 16x256b.x2 load without the wait: 16 lanes x 16 columns, as above with two
-// 8-column groups.
 __device__ __forceinline__ void tmem_ld16x256_x2_nowait(uint32_t taddr, uint32_t* r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
