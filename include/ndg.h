@@ -379,6 +379,15 @@ ndg_status ndg_forward_batch(const ndg_frame* frames, int n_frames, void* batch_
  * word is used). */
 ndg_status ndg_selftest_timeout(int which, void* ws, size_t ws_bytes, ndg_stream stream);
 
+/* Accuracy self-test of the preparation's FP64 functions: evaluates each at
+ * a[i] with the library's own code (own [n]) and with CUDA's exp() and
+ * division (cuda [n]).  which = 0: exp(v); 1: 1 / (1 + exp(-v)); 2:
+ * 2 / (1 + exp(-v)) - 1 (v = a[i] rounded to FP32); 3: a[i] / b[i], both of
+ * magnitude 2^-400 to 2^400 (b is unused otherwise and may be NULL).  Device
+ * arrays, 8-byte aligned. */
+ndg_status ndg_selftest_math(int which, long long n, const double* a, const double* b,
+                             double* own, double* cuda, ndg_stream stream);
+
 /* Measurement helper (no counterpart in the paper): throughput probe of one
  * arithmetic pipe, for the rooflines the benchmark reports.  which = 0: the
  * MUFU exponential (ex2.approx, one per Gaussian-query pair in every

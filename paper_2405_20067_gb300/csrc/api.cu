@@ -604,6 +604,16 @@ ndg_status ndg_selftest_timeout(int which, void* ws, size_t ws_bytes, ndg_stream
   return cuda_ok();
 }
 
+ndg_status ndg_selftest_math(int which, long long n, const double* a, const double* b,
+                             double* own, double* cuda, ndg_stream stream) {
+  if (which < 0 || which > 3 || n < 0) return NDG_ERR_INVALID_ARG;
+  if (n > 0 && (!a || !own || !cuda || (which == 3 && !b))) return NDG_ERR_INVALID_ARG;
+  if (!aligned(a, 8) || !aligned(b, 8) || !aligned(own, 8) || !aligned(cuda, 8))
+    return NDG_ERR_INVALID_ARG;
+  launch_selftest_math(which, n, a, b, own, cuda, (cudaStream_t)stream);
+  return cuda_ok();
+}
+
 namespace {
 
 // Gaussian-major order of the entries (the stable order of a sort by

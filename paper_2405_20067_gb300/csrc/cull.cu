@@ -22,6 +22,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "kernels.h"
+#include "prep_math.cuh"
 
 namespace ndg {
 
@@ -115,62 +116,9 @@ __global__ void tile_keys_kernel(const float* __restrict__ tb, long long T, int 
 }
 
 // ---- prep: activation, prepared record, Gaussian keys --------------------------
-// The preparation is bound by FP64 arithmetic (two lanes per clock and SM), so
-// its exponentials and reciprocals are written for FP32 arguments and ordinary
-// ranges with as few FP64 operations as double precision takes.
-//
-// exp(v) by table and polynomial: k = round(64 v / ln 2) (from FP32, any
-// nearby integer does), r = v - k ln2 / 64 with ln2 / 64 split so that
-// k * high part is exact, exp(v) = 2^(k / 64) (1 + r + ... + r^5 / 120), the
-// remainder r^6 / 720 below 4e-17 for |r| <= ln2 / 128.  Within 1 ulp; 9 FP64
-// operations and 2 conversions.  Arguments whose result leaves the normal
-// range go to exp().
-__device__ const double kExp2Table[64] = {  // 2^(j / 64)
-    0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
-    0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0, 0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0,
-    0x1.172b83c7d517bp+0, 0x1.1a35beb6fcb75p+0, 0x1.1d4873168b9aap+0, 0x1.2063b88628cd6p+0,
-    0x1.2387a6e756238p+0, 0x1.26b4565e27cddp+0, 0x1.29e9df51fdee1p+0, 0x1.2d285a6e4030bp+0,
-    0x1.306fe0a31b715p+0, 0x1.33c08b26416ffp+0, 0x1.371a7373aa9cbp+0, 0x1.3a7db34e59ff7p+0,
-    0x1.3dea64c123422p+0, 0x1.4160a21f72e2ap+0, 0x1.44e086061892dp+0, 0x1.486a2b5c13cd0p+0,
-    0x1.4bfdad5362a27p+0, 0x1.4f9b2769d2ca7p+0, 0x1.5342b569d4f82p+0, 0x1.56f4736b527dap+0,
-    0x1.5ab07dd485429p+0, 0x1.5e76f15ad2148p+0, 0x1.6247eb03a5585p+0, 0x1.6623882552225p+0,
-    0x1.6a09e667f3bcdp+0, 0x1.6dfb23c651a2fp+0, 0x1.71f75e8ec5f74p+0, 0x1.75feb564267c9p+0,
-    0x1.7a11473eb0187p+0, 0x1.7e2f336cf4e62p+0, 0x1.82589994cce13p+0, 0x1.868d99b4492edp+0,
-    0x1.8ace5422aa0dbp+0, 0x1.8f1ae99157736p+0, 0x1.93737b0cdc5e5p+0, 0x1.97d829fde4e50p+0,
-    0x1.9c49182a3f090p+0, 0x1.a0c667b5de565p+0, 0x1.a5503b23e255dp+0, 0x1.a9e6b5579fdbfp+0,
-    0x1.ae89f995ad3adp+0, 0x1.b33a2b84f15fbp+0, 0x1.b7f76f2fb5e47p+0, 0x1.bcc1e904bc1d2p+0,
-    0x1.c199bdd85529cp+0, 0x1.c67f12e57d14bp+0, 0x1.cb720dcef9069p+0, 0x1.d072d4a07897cp+0,
-    0x1.d5818dcfba487p+0, 0x1.da9e603db3285p+0, 0x1.dfc97337b9b5fp+0, 0x1.e502ee78b3ff6p+0,
-    0x1.ea4afa2a490dap+0, 0x1.efa1bee615a27p+0, 0x1.f50765b6e4540p+0, 0x1.fa7c1819e90d8p+0};
-__device__ __forceinline__ double exp_f32(float v) {
-  if (!(fabsf(v) < 700.0f)) return exp((double)v);
-  const float kf = rintf(v * 92.33248261689366f);
-  const int k = (int)kf;
-  const double kd = (double)kf;
-  double r = fma(kd, -0x1.62e42fee00000p-7, (double)v);
-  r = fma(kd, -0x1.a39ef35793c76p-39, r);
-  double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-  q = fma(q, r, 1.0 / 6.0);
-  q = fma(q, r, 0.5);
-  q = fma(q * r, r, r);
-  const double t = __ldg(kExp2Table + (k & 63));
-  const double e = fma(t, q, t);
-  return __hiloint2double(__double2hiint(e) + ((k >> 6) << 20), __double2loint(e));
-}
-// 1 / d for 1 <= d: the approximate reciprocal (2^-20 or better) and one cubic
-// correction x (1 + e + e^2), e = 1 - d x.
-__device__ __forceinline__ double rcp_ge1(double d) {
-  if (!(d < 1e300)) return 1.0 / d;
-  double x;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
-  double e = fma(-d, x, 1.0);
-  e = fma(e, e, e);
-  return fma(e, x, x);
-}
-
 // Section 3.1 (Eq. 2): L_ii = exp(theta_ii), L_ij = 2 sigmoid(theta_ij) - 1;
-// evaluated in FP64 and rounded once to FP32 so that the FP32 values that
-// feed the cull contract are the correctly rounded activations.
+// evaluated in FP64 and rounded once to FP32 for the cull contract (2 sigmoid
+// - 1 carries an absolute error of up to 3.4e-16, as the plain formula does).
 template <int N>
 __device__ __forceinline__ void act_lower64(const float* __restrict__ th, double* L) {
 #pragma unroll
@@ -178,7 +126,7 @@ __device__ __forceinline__ void act_lower64(const float* __restrict__ th, double
 #pragma unroll
     for (int j = 0; j <= i; ++j) {
       const float v = th[tri(i) + j];
-      L[tri(i) + j] = (i == j) ? exp_f32(v) : fma(2.0, rcp_ge1(1.0 + exp_f32(-v)), -1.0);
+      L[tri(i) + j] = (i == j) ? exp_f32(v) : off_diagonal(v);
     }
 }
 
@@ -347,7 +295,7 @@ __global__ void __launch_bounds__(32) prep_kernel(PrepArgs a) {
   bool finite = true;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    wf[c] = (float)(alpha * rcp_ge1(1.0 + exp_f32(-gam[c])));
+    wf[c] = (float)(alpha * sigmoid(gam[c]));
     finite &= isfinite(wf[c]);
   }
   float Lf[P], mf[N];
@@ -358,8 +306,8 @@ __global__ void __launch_bounds__(32) prep_kernel(PrepArgs a) {
   if (!finite && a.status) set_status(a.status, NDG_ERR_NUMERIC);
 
   if (a.rec) {
-    // M = L^{-1} (lower) by forward substitution on the identity, in FP64.
-    // The rows' divisions share one reciprocal each.
+    // M = L^{-1} (lower) by forward substitution on the identity, in FP64; a
+    // row's quotients share its diagonal's reciprocal.
     double M[P];
 #pragma unroll
     for (int j = 0; j < N; ++j) M[tri(j) + j] = 1.0 / L[tri(j) + j];
@@ -370,7 +318,7 @@ __global__ void __launch_bounds__(32) prep_kernel(PrepArgs a) {
         double s = 0.0;
 #pragma unroll
         for (int kk = j; kk < i; ++kk) s = fma(L[tri(i) + kk], M[tri(kk) + j], s);
-        M[tri(i) + j] = -s * M[tri(i) + i];
+        M[tri(i) + j] = quotient(-s, L[tri(i) + i], M[tri(i) + i]);
       }
     }
     float* out = a.rec + (size_t)e * (a.rec_kind == 2 ? rec_tc_floats(N) : R);

@@ -151,6 +151,8 @@ int launch_loss(const float* y, const float* target, float* dy, long long n, dou
                 double* loss, cudaStream_t s, double rel_eps = -1.0, long long norm = 0);
 int launch_bwd(int N, const BwdArgs& a, long long T, cudaStream_t s);
 int launch_selftest_wait(int* status, int which, cudaStream_t s);
+int launch_selftest_math(int which, long long n, const double* a, const double* b, double* own,
+                         double* cuda, cudaStream_t s);
 int launch_segsum(const float* part, int RP, const long long* goff, int Ge, const int32_t* perm,
                   long long n_cap, int* status, float* gsum, cudaStream_t s);
 int launch_chain(int N, const ChainArgs& a, cudaStream_t s);

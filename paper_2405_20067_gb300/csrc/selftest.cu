@@ -3,11 +3,13 @@
 // completes, with the same wait helpers as the tensor-core kernels.  When
 // the bound runs out the CTA records NDG_ERR_TIMEOUT in the workspace status
 // word and returns, so the context stays usable; nothing faults or traps.
+// And the preparation's FP64 functions beside CUDA's (ndg_selftest_math).
 #include <cuda_runtime.h>
 
 #include "common.cuh"
 #include "internal.h"
 #include "kernels.h"
+#include "prep_math.cuh"
 #include "tcgen05.cuh"
 
 namespace ndg {
@@ -39,6 +41,37 @@ __global__ void selftest_wait_kernel(int* status, int which) {
 
 int launch_selftest_wait(int* status, int which, cudaStream_t s) {
   selftest_wait_kernel<<<1, 64, 0, s>>>(status, which);
+  return 1;
+}
+
+// Functions as in prep_math.cuh; arguments of 0 to 2 are rounded to FP32.
+__global__ void selftest_math_kernel(int which, long long n, const double* __restrict__ a,
+                                     const double* __restrict__ b, double* __restrict__ own,
+                                     double* __restrict__ cuda) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const float v = (float)a[i];
+    if (which == 0) {
+      own[i] = exp_f32(v);
+      cuda[i] = exp((double)v);
+    } else if (which == 1) {
+      own[i] = sigmoid(v);
+      cuda[i] = 1.0 / (1.0 + exp(-(double)v));
+    } else if (which == 2) {
+      own[i] = off_diagonal(v);
+      cuda[i] = 2.0 / (1.0 + exp(-(double)v)) - 1.0;
+    } else {
+      own[i] = quotient(a[i], b[i], 1.0 / b[i]);
+      cuda[i] = a[i] / b[i];
+    }
+  }
+}
+
+int launch_selftest_math(int which, long long n, const double* a, const double* b, double* own,
+                         double* cuda, cudaStream_t s) {
+  if (n <= 0) return 0;
+  const long long blocks = ceil_div<long long>(n, 256);
+  selftest_math_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(which, n, a, b, own, cuda);
   return 1;
 }
 

@@ -108,7 +108,7 @@ def _tr(trace):
 EXPORTS = ["ndg_workspace_size", "ndg_build_cull", "ndg_build_cull_conditioned", "ndg_forward",
            "ndg_loss_l2", "ndg_loss_rel_l2", "ndg_backward", "ndg_adam", "ndg_densify",
            "ndg_read_status", "ndg_status_string", "ndg_version", "ndg_forward_noalloc",
-           "ndg_selftest_timeout", "ndg_probe_pipe", "ndg_loss_l2_shard",
+           "ndg_selftest_timeout", "ndg_selftest_math", "ndg_probe_pipe", "ndg_loss_l2_shard",
            "ndg_batch_workspace_size", "ndg_forward_batch", "ndg_backward_order"]
 NDG_ERR_SCRATCH_LIMIT = 7
 
@@ -145,6 +145,7 @@ def lib():
         L.ndg_batch_workspace_size.restype = sz
         L.ndg_forward_batch.argtypes = [ctypes.POINTER(FrameC), ctypes.c_int, _P, sz, _P, _P, TR]
         L.ndg_selftest_timeout.argtypes = [ctypes.c_int, _P, sz, _P]
+        L.ndg_selftest_math.argtypes = [ctypes.c_int, ctypes.c_longlong, _P, _P, _P, _P, _P]
         L.ndg_probe_pipe.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, _P,
                                      _P, _P]
         L.ndg_read_status.argtypes = [_P, _P, ctypes.POINTER(ctypes.c_int)]
@@ -154,7 +155,7 @@ def lib():
         for name in ["ndg_build_cull", "ndg_build_cull_conditioned", "ndg_forward", "ndg_loss_l2",
                      "ndg_loss_rel_l2", "ndg_backward", "ndg_adam", "ndg_densify",
                      "ndg_read_status", "ndg_forward_noalloc", "ndg_selftest_timeout",
-                     "ndg_probe_pipe", "ndg_loss_l2_shard", "ndg_forward_batch",
+                     "ndg_selftest_math", "ndg_probe_pipe", "ndg_loss_l2_shard", "ndg_forward_batch",
                      "ndg_backward_order"]:
             getattr(L, name).restype = ctypes.c_int
         _lib = L
@@ -388,6 +389,16 @@ def selftest_timeout(which: int, ws: torch.Tensor, stream=None):
     records NDG_ERR_TIMEOUT in the workspace status word (read_status)."""
     _check(lib().ndg_selftest_timeout(int(which), _ptr(ws), ws.numel(), _stream(stream)),
            "ndg_selftest_timeout")
+
+
+def selftest_math(which: int, a: torch.Tensor, b: torch.Tensor | None = None, stream=None):
+    """The preparation's FP64 functions (0: exp, 1: sigmoid, 2: 2 sigmoid - 1,
+    3: a / b) at FP64 arguments: (the library's own values, CUDA's)."""
+    assert a.is_cuda and a.dtype == torch.float64 and a.is_contiguous()
+    own, cuda = torch.empty_like(a), torch.empty_like(a)
+    _check(lib().ndg_selftest_math(int(which), a.numel(), _ptr(a), _ptr(b), _ptr(own), _ptr(cuda),
+                                   _stream(stream)), "ndg_selftest_math")
+    return own, cuda
 
 
 def probe_pipe(which: int, reps: int = 5, iters: int = 2048, threads: int = 1024) -> dict:
