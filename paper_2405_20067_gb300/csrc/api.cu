@@ -29,6 +29,15 @@ namespace ndg {
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
+// SMs of the current device; 0 if the query fails.
+static int sm_count() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
+  return sms;
+}
+
 ndg_status check_mix(const ndg_mixture* m) {
   if (!m) return NDG_ERR_INVALID_ARG;
   if (m->N < 1 || m->N > NDG_MAX_N || m->G < 0 || m->G_cap < m->G) return NDG_ERR_INVALID_ARG;
@@ -482,10 +491,8 @@ ndg_status ndg_forward_batch(const ndg_frame* frames, int n_frames, void* batch_
     if (fr.flags & ~NDG_RECORDS_READY) return NDG_ERR_INVALID_ARG;
   }
   // one persistent CTA per SM (queried before anything is launched)
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-    return NDG_ERR_CUDA;
+  const int sms = sm_count();
+  if (sms < 1) return NDG_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
   Tracer tr(trace, s);
   std::vector<char> img(bl.end, 0);
@@ -687,6 +694,8 @@ ndg_status ndg_backward(const ndg_mixture* mix, const ndg_queries* q, const ndg_
       (st = check_mix(grad)))
     return st ? st : NDG_ERR_INVALID_ARG;
   if (q->Q > 0 && !dy) return NDG_ERR_INVALID_ARG;
+  const int sms = sm_count();
+  if (sms < 1) return NDG_ERR_CUDA;
   Sizes z = make_sizes(mix, q, nullptr, cull->E_cap);
   CommonLayout c = common_layout(z);
   BwdLayout L = bwd_layout(z, c.end);
@@ -715,6 +724,8 @@ ndg_status ndg_backward(const ndg_mixture* mix, const ndg_queries* q, const ndg_
   ba.Ge = pa.Ge;
   ba.slot = nullptr;
   ba.part = (float*)(w + L.part);
+  ba.E_cap = cull->E_cap;
+  ba.sms = sms;
   ba.status = pa.status;
   tr.begin();
   // tensor cores: the E Psi form for N <= 6, the beta form (bwd_hb.cu) above

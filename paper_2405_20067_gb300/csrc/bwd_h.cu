@@ -175,10 +175,14 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long t = blockIdx.x;
+  __shared__ long long s_range[2];  // this part's entries, read again after the setup
   {
     long long b = a.offsets[t], e = a.offsets[t + 1];
-    part_range(b, e, NC);
-    if (b >= e) return;
+    if (!part_of_list(b, e, a.sms, kSplitPsi)) return;
+    if (tid == 0) {
+      s_range[0] = b;
+      s_range[1] = e;
+    }
   }
   const long long qt = t * a.tile;
   const int nq = (int)(a.Q - qt < a.tile ? a.Q - qt : a.tile);
@@ -286,8 +290,7 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = tmem_base;
-  long long beg = a.offsets[t], end = a.offsets[t + 1];
-  part_range(beg, end, NC);
+  const long long beg = s_range[0], end = s_range[1];
   const int nchunks = (int)((end - beg + NC - 1) / NC);
   const int U = nchunks * nh;
   volatile int* abort_flag = &s_abort;
@@ -661,7 +664,7 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
 
 int launch_bwd_h(int N, const BwdArgs& a, long long T, cudaStream_t s) {
   if (T <= 0) return 0;
-  const dim3 grid((unsigned)T, (unsigned)split_parts(N, T, kSMs));  // one CTA per SM
+  const dim3 grid((unsigned)T, (unsigned)launch_parts(T, a.E_cap, a.sms, kSplitPsi, true));
 #define L_BH(n)                                                                         \
   {                                                                                     \
     cudaFuncSetAttribute(bwd_h_kernel<n>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \

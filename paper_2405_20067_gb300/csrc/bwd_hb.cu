@@ -190,9 +190,15 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long t = blockIdx.x;
-  long long beg = a.offsets[t], end = a.offsets[t + 1];
-  part_range(beg, end, NC);
-  if (beg >= end) return;
+  __shared__ long long s_range[2];  // this part's entries, read again after the setup
+  {
+    long long b = a.offsets[t], e = a.offsets[t + 1];
+    if (!part_of_list(b, e, a.sms, kSplitBeta)) return;
+    if (tid == 0) {
+      s_range[0] = b;
+      s_range[1] = e;
+    }
+  }
   const long long qt = t * a.tile;
   const int nq = (int)(a.Q - qt < a.tile ? a.Q - qt : a.tile);
   const int nh = (nq + S::UQ - 1) / S::UQ;  // units per chunk
@@ -303,6 +309,7 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = tmem_base;
+  const long long beg = s_range[0], end = s_range[1];
   const int nchunks = (int)((end - beg + NC - 1) / NC);
   const int U = nchunks * nh;
   volatile int* abort_flag = &s_abort;
@@ -792,7 +799,7 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
 
 int launch_bwd_hb(int N, const BwdArgs& a, long long T, cudaStream_t s) {
   if (T <= 0) return 0;
-  const dim3 grid((unsigned)T, (unsigned)split_parts(N, T, kSMs));  // one CTA per SM
+  const dim3 grid((unsigned)T, (unsigned)launch_parts(T, a.E_cap, a.sms, kSplitBeta, true));
 #define L_BB(n)                                                                         \
   {                                                                                     \
     cudaFuncSetAttribute(bwd_hb_kernel<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, \

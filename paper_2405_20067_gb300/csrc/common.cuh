@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "ndg.h"
+#include "split.h"
 
 namespace ndg {
 
@@ -54,33 +55,28 @@ __device__ __forceinline__ int clampi(int v, int a, int b) { return v < a ? a : 
 template <typename T>
 __host__ __device__ inline T ceil_div(T a, T b) { return (a + b - 1) / b; }
 
-// ---- several CTAs per tile in the backward -------------------------------------
-// An entry's record depends on its own Gaussian and the tile's queries alone,
-// so a tile's candidates may be split over CTAs (grid y) without changing a
-// bit.  Few tiles leave SMs idle and a last wave nearly empty; every part pays
-// the tile's setup again, taken as 1/25 of an average tile, and as 1/5 for
-// N < 6, whose tiles are cheap (N = 3, 512 tiles: two parts, which 1/25 would
-// choose, measured 119 us against 109 to 114 for one).  slots: CTAs resident on the chip.  Measured:
-// N = 6, 16 tiles 406 -> 42 us, N = 6 FP32, 64 tiles 128 -> 52 us and 1,024
-// tiles 5.20 -> 4.31 ms, N = 10, 63 tiles of 128 queries 318 -> 138 us (start
-// against now, other changes of the TC kernels included).
-constexpr int kSMs = 152;
-inline int split_parts(int N, long long T, int slots) {
-  int best = 1;
-  double cost = 1e30;
-  const double setup = N < 6 ? 0.2 : 0.04;
-  for (int S = 1; S <= 8; ++S) {
-    const double c = (double)ceil_div<long long>(T * S, slots) * (1.0 / S + setup);
-    if (c < cost) { cost = c; best = S; }
+// ---- several CTAs per tile in the backward (split.h) ----------------------------
+// Part p of S of entries [beg, end), in steps of `step`; false if empty.
+__device__ __forceinline__ bool part_of(long long& beg, long long& end, int step, int p, int S) {
+  if (S > 1) {
+    const long long n = (end - beg + step - 1) / step;
+    const long long e = beg + n * (p + 1) / S * step;
+    beg += n * p / S * step;
+    end = e < end ? e : end;
   }
-  return best;
+  return beg < end;
 }
-// The part blockIdx.y of gridDim.y of entries [beg, end), in steps of `step`.
-__device__ __forceinline__ void part_range(long long& beg, long long& end, int step) {
-  const long long n = (end - beg + step - 1) / step, p = blockIdx.y, S = gridDim.y;
-  const long long e = beg + n * (p + 1) / S * step;
-  beg += n * p / S * step;
-  end = e < end ? e : end;
+// The same for CTA blockIdx.y of a tile that its own list splits into at most
+// gridDim.y parts.
+__device__ __forceinline__ bool part_of_list(long long& beg, long long& end, int sms, SplitCost k) {
+  int S = 1;
+  if (gridDim.y > 1) {
+    const long long n = (end - beg + k.step - 1) / k.step;
+    if (gridDim.x * gridDim.y <= (unsigned)sms) S = n < gridDim.y ? (int)n : (int)gridDim.y;  // one wave
+    else S = split_parts(gridDim.x, (unsigned)(n < kMaxSteps ? n : kMaxSteps), gridDim.y, (unsigned)sms, k, false);
+  }
+  const int p = blockIdx.y;
+  return p < S && part_of(beg, end, k.step, p, S);
 }
 
 // ---- tile centre ---------------------------------------------------------------

@@ -86,6 +86,8 @@ struct BwdArgs {
   int* status;               // device status word (timeouts of bounded waits)
   const int32_t* slot;       // entry -> output record index, or null (entry order)
   float* part;               // [E_cap][part_floats(N)]
+  long long E_cap;           // capacity of the lists, and the device's SMs: they
+  int sms;                   // choose the CTAs per tile (split.h)
 };
 
 struct ChainArgs {
