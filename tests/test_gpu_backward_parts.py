@@ -1,10 +1,12 @@
 """The backward with a tile's candidates in several parts and in one: the same
-bits, at list lengths on both sides of the chunks' and the parts' edges.  A launch of a few tiles is split; the same tiles
+bits, at list lengths on both sides of the chunks' and the parts' edges; and
+lists of many chunks in one CTA against the oracle (the reuse of every stage,
+stash slot and accumulator).  A launch of a few tiles is split; the same tiles
 followed by empty ones are not (the rule goes by the average list)."""
 import numpy as np
 import pytest
 
-from helpers import NAMES
+from helpers import NAMES, assert_grads_close, oracle_raw
 from paper_2405_20067_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -71,3 +73,17 @@ def test_parts_give_the_bits_of_one(ndg, N, mode):
     roomy = backward(ndg, N, mix, x[:T * TILE], dy[:T * TILE], offs[:T + 1], ids, md, cap=40 * len(ids))
     for n, a, b in zip(NAMES, roomy, whole):
         assert np.array_equal(a, b), n
+
+
+@pytest.mark.parametrize("N", [3, 6, 7, 8, 9, 10, 11, 12])
+def test_many_chunks_in_one_cta_match_the_oracle(ndg, oracle, N):
+    """10 chunks of two query units and 7 of one (a tile of 100 queries last)."""
+    lengths, G = [9 * 128 + 5, 7 * 128 - 3], 1300
+    mix, x, dy = inputs(N, G, 2, EMPTY, 600 + N)
+    # the short tile last: the empty tiles come first
+    x, dy = np.roll(x, EMPTY * TILE, axis=0)[:-156], np.roll(dy, EMPTY * TILE, axis=0)[:-156]
+    offs, ids = lists(G, lengths, 0, 610 + N)
+    offs = np.concatenate([np.zeros(EMPTY, np.int64), offs])
+    got = dict(zip(NAMES, backward(ndg, N, mix, x, dy, offs, ids, ndg.NDG_MODE_TC)))
+    want = oracle.grad(oracle_raw(oracle, mix), x.astype(np.float64), TILE, offs, ids, dy.astype(np.float64))
+    assert_grads_close(got, want, NAMES[:4], rtol=1e-3)
