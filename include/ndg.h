@@ -370,10 +370,11 @@ ndg_status ndg_forward_batch(const ndg_frame* frames, int n_frames, void* batch_
                              ndg_stream stream, ndg_trace* trace);
 
 /* Failure-detection self-test of the bounded device waits: launches one
- * CTA that waits on an mbarrier nothing ever completes, with the wait the
- * tensor-core kernels use (which = 0: the roles' warp wait, about a
- * second; which = 1: the spinning wait of their final drain, about a second
- * or two).  When the bound runs out it records NDG_ERR_TIMEOUT in the
+ * CTA that waits on an mbarrier nothing ever completes, with the waits the
+ * tensor-core kernels use (which = 0: the roles' waits, a warp's and the MMA
+ * issuer's single lane, about a second; which = 1: the spinning wait of their
+ * final drain, about five seconds).  When the bounds run out, none of them
+ * within 0.2 s, it records NDG_ERR_TIMEOUT in the
  * workspace status word (read with ndg_read_status) and returns; nothing
  * faults and the context stays usable.  ws: any workspace (only its status
  * word is used). */

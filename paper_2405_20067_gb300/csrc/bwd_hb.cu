@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
       constexpr uint64_t PHI_LO = S::LO_OFF >> 4, C_LO = S::C_BYTES >> 4;
       auto mma1 = [&](int u) -> bool {
         const int i = u / nh, h = u - i * nh, s = i % CS, sb = u % NBUF;
-        if (h == 0 && !mbar_wait_abort(&coef_full[s], (i / CS) & 1, abort_flag)) return false;
+        if (h == 0 && !lane_wait(&coef_full[s], (i / CS) & 1, abort_flag)) return false;
         fence_after_sync();
         const uint64_t dch = dC0 + (uint64_t)((s * S::C_STAGE) >> 4);
         const uint64_t dph = dPhiK + (uint64_t)((h * 16 * S::GRP) >> 4);  // 16 groups per unit
@@ -506,8 +506,8 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
       };
       auto mma2 = [&](int u) -> bool {
         const int i = u / nh, h = u - i * nh, sb = u % NBUF, db = i & 1;
-        if (!mbar_wait_abort(&e_full[sb], (u / NBUF) & 1, abort_flag)) return false;
-        if (h == 0 && i >= 2 && !mbar_wait_abort(&d_empty[db], ((i >> 1) - 1) & 1, abort_flag))
+        if (!lane_wait(&e_full[sb], (u / NBUF) & 1, abort_flag)) return false;
+        if (h == 0 && i >= 2 && !lane_wait(&d_empty[db], ((i >> 1) - 1) & 1, abort_flag))
           return false;
         fence_after_sync();
         const uint32_t d = tmem + S::TM_D + (uint32_t)(db * ND);

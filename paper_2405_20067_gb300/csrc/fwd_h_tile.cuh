@@ -487,11 +487,11 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& a, long long t) {
       constexpr uint32_t IDESC = idesc_f16(NC);
       for (int i = 0; i < nchunks; ++i) {
         const int s = i % CS, b = i & 1;
-        bool ok = mbar_wait_abort(&coef_full[s], (i / CS) & 1, abort_flag);
+        bool ok = lane_wait(&coef_full[s], (i / CS) & 1, abort_flag);
         const uint64_t dbh = dB0 + (uint64_t)((s * S::C_STAGE) >> 4);
         for (int h = 0; ok && h < nh; ++h) {
           // row block h of buffer b is free once its epilogue group has read chunk i - 2
-          if (i >= 2) ok = mbar_wait_abort(&acc_empty[2 * b + h], ((i >> 1) - 1) & 1, abort_flag);
+          if (i >= 2) ok = lane_wait(&acc_empty[2 * b + h], ((i >> 1) - 1) & 1, abort_flag);
           if (!ok) break;
           fence_after_sync();
           const uint32_t d = tmem + (uint32_t)((2 * b + h) * NC);

@@ -14,20 +14,30 @@
 
 namespace ndg {
 
-// which = 0: the roles' warp wait (warp_wait: every lane polls, kPollLimit
-// polls); which = 1: the spinning wait of the
-// kernels' final drain (mbar_wait_bounded, kWaitLimit polls).
+__device__ __forceinline__ unsigned long long selftest_ns() {
+  unsigned long long v;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(v));
+  return v;
+}
+
+// which = 0: the roles' waits, a warp's (warp_wait) by warp 0 and the issuer's
+// (lane_wait) by a lane of warp 1 at the same time; which = 1: the spinning
+// wait of the kernels' final drain (mbar_wait_bounded, kWaitLimit polls).  The
+// timeout is recorded if every wait ran out, none of them within 0.2 s (a
+// shorter bound would end kernels that are only delayed).
 __global__ void selftest_wait_kernel(int* status, int which) {
   __shared__ uint64_t bar;
-  __shared__ int abort_flag;
+  __shared__ int abort_flag, good;
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);  // one arrival expected; none is ever made
     abort_flag = 0;
+    good = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  const unsigned long long t0 = selftest_ns();
+  bool ok = true;
   if (threadIdx.x < 32) {
-    bool ok;
     if (which == 0) {
       ok = warp_wait(&bar, 0, &abort_flag);
     } else {
@@ -35,8 +45,16 @@ __global__ void selftest_wait_kernel(int* status, int which) {
       if (threadIdx.x == 0) r = mbar_wait_bounded(&bar, 0, kWaitLimit) ? 1 : 0;
       ok = __shfl_sync(0xffffffffu, r, 0) != 0;
     }
-    if (!ok && threadIdx.x == 0 && status) set_status(status, NDG_ERR_TIMEOUT);
+  } else if (which == 0) {
+    int r = 1;
+    if (threadIdx.x == 32) r = lane_wait(&bar, 0, &abort_flag) ? 1 : 0;
+    ok = __shfl_sync(0xffffffffu, r, 0) != 0;
   }
+  const bool waited = which == 0 || threadIdx.x < 32;
+  if ((threadIdx.x & 31) == 0 && (!waited || (!ok && selftest_ns() - t0 >= 200000000ull)))
+    atomicAdd(&good, 1);
+  __syncthreads();
+  if (threadIdx.x == 0 && good == 2 && status) set_status(status, NDG_ERR_TIMEOUT);
 }
 
 int launch_selftest_wait(int* status, int which, cudaStream_t s) {

@@ -166,6 +166,7 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
          ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
 }
 
+// Polls of the final drain's wait (one lane, 70 to 85 ns each: about 5 s).
 constexpr uint32_t kWaitLimit = 1u << 26;
 
 // kind::f16 MMA (FP16 A and B, FP32 accumulator in TMEM).
@@ -184,24 +185,31 @@ __host__ __device__ constexpr uint32_t idesc_f16(int n) {
   return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
 }
 
-// Bounded wait that gives up once another thread has raised *abort (a poll
-// takes ~3.8 us when the phase does not complete: at most ~1 s).
-constexpr uint32_t kPollLimit = 1u << 18;
+// Bounded wait that gives up once another thread has raised *abort.
 __device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, uint32_t parity,
-                                                volatile int* abort) {
-  for (uint32_t i = 0; i < kPollLimit; ++i) {
+                                                volatile int* abort, uint32_t polls) {
+  for (uint32_t i = 0; i < polls; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if (*abort) return false;
   }
   return false;
 }
 
+// The issuer's wait, by one lane: a poll of a phase that does not complete
+// takes 97 ns, so that it gives up after 0.8 s.
+constexpr uint32_t kLanePolls = 1u << 23;
+__device__ __forceinline__ bool lane_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  return mbar_wait_abort(bar, parity, abort, kLanePolls);
+}
+
 // Warp-level bounded wait: every lane polls for itself and the warp leaves
 // together.  (Lane 0 polling, with a suspend-time hint, and handing its
 // outcome on by a shuffle cost ~600 cycles per wait, also on a completed
-// phase: N = 6 backward 33.4 -> 24.2 ms.)
+// phase: N = 6 backward 33.4 -> 24.2 ms.)  A warp's poll takes 3.8 us: it
+// gives up after 1 s.
+constexpr uint32_t kWarpPolls = 1u << 18;
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  const bool ok = mbar_wait_abort(bar, parity, abort);
+  const bool ok = mbar_wait_abort(bar, parity, abort, kWarpPolls);
   return __all_sync(0xffffffffu, ok);
 }
 

@@ -48,3 +48,20 @@ def test_wait_on_a_barrier_nothing_completes_times_out(ndg, oracle, which):
     yo = oracle.eval(L, m, w, x.astype(np.float64), tile, offs, ids)
     assert_outputs_close(y, yo, rtol=1e-3, floor=1e-3)
     assert ndg.read_status(ev.ws) == 0
+
+
+@pytest.mark.parametrize("which", [0, 1])
+def test_waits_give_up_in_time_but_not_at_once(ndg, which):
+    """Every kind of wait holds for at least 0.2 s (the self-test reports no
+    timeout for one that ends sooner) and all end within ten."""
+    import torch
+    ws = ndg.workspace(1 << 16)
+    begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda.synchronize()
+    begin.record()
+    ndg.selftest_timeout(which, ws)
+    end.record()
+    assert ndg.read_status(ws) == NDG_ERR_TIMEOUT
+    s = begin.elapsed_time(end) * 1e-3
+    print(f"waits {which}: {s:.2f} s")
+    assert 0.2 < s < 10.0
