@@ -290,6 +290,8 @@ ndg_status build_cull(const ndg_mixture* mix, const ndg_queries* q, const ndg_cu
   CommonLayout c = common_layout(z);
   CullLayout L = cull_layout(z, c.end);
   if (ws_bytes < L.end) return NDG_ERR_WORKSPACE;
+  const int sms = sm_count();
+  if (sms < 1) return NDG_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
   Tracer tr(trace, s);
   char* w = (char*)ws;
@@ -345,6 +347,7 @@ ndg_status build_cull(const ndg_mixture* mix, const ndg_queries* q, const ndg_cu
   ca.E_cap = out->E_cap;
   ca.masks = (uint32_t*)(w + L.masks);
   ca.mask_words = mask_words(z);
+  ca.sms = sms;
   tr += launch_cull_tile(KP, ca, T, s);
   long long* excl = (long long*)(w + L.excl);
   tr += scan_exclusive_i64(ca.counts, excl, 8 * T, w + L.tmp, s);

@@ -691,16 +691,16 @@ int launch_permute_keys(const uint8_t* src, const int32_t* sorted, int n, int KP
 
 // Tiles per CTA of the count pass: four while that still gives every SM four
 // CTAs (a key row is then read once for four tiles), fewer for few tiles.
-int cull_group(int KP, long long T) {
+int cull_group(int KP, long long T, int sms) {
   if (KP == 0) return 1;
-  return T >= 4 * 4 * 152 ? 4 : T >= 2 * 4 * 152 ? 2 : 1;
+  return T >= 4 * 4ll * sms ? 4 : T >= 2 * 4ll * sms ? 2 : 1;
 }
 
 int launch_cull_tile(int KP, const CullTileArgs& args, long long T, cudaStream_t s) {
   if (T <= 0) return 0;
   CullTileArgs a = args;
   a.T = T;
-  a.group = cull_group(KP, T);
+  a.group = cull_group(KP, T, a.sms);
   const unsigned groups = (unsigned)ceil_div<long long>(T, a.group);
   const bool small = a.B <= 128;
 #define L_CC(K, TG)                                                          \

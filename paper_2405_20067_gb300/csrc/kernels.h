@@ -42,6 +42,7 @@ struct CullTileArgs {
   long long mask_words;       // per tile: >= ceil(max sources / 32) + 8
   long long T;                // set by launch_cull_tile: tiles, and tiles per
   int group;                  // CTA of the count pass
+  int sms;                    // SMs of the device
 };
 
 struct FwdArgs {
