@@ -1,6 +1,6 @@
 // bwd_hb.cu -- the analytic backward on the tensor cores in the beta form
-// (ndg_backward, NDG_MODE_TC, N = 7..12; built for every N <= 12, while
-// N <= 6 dispatches the E Psi form of bwd_h.cu, measured faster there).
+// (ndg_backward, NDG_MODE_TC, N = 7..12; N <= 6 takes the E Psi form of
+// bwd_h.cu).
 //
 // With the lifted form of the forward (s = phi(x~) . coef, e = 2^s, the
 // coefficients scaled by -log2(e) / 2), the gradients of an entry (Gaussian
@@ -807,12 +807,6 @@ int launch_bwd_hb(int N, const BwdArgs& a, long long T, cudaStream_t s) {
     bwd_hb_kernel<n><<<grid, 416, BwdBShape<n>::SMEM, s>>>(a);                   \
   }
   switch (N) {
-    case 1: L_BB(1); break;
-    case 2: L_BB(2); break;
-    case 3: L_BB(3); break;
-    case 4: L_BB(4); break;
-    case 5: L_BB(5); break;
-    case 6: L_BB(6); break;
     case 7: L_BB(7); break;
     case 8: L_BB(8); break;
     case 9: L_BB(9); break;

@@ -713,7 +713,10 @@ int launch_cull_tile(int KP, const CullTileArgs& args, long long T, cudaStream_t
   else { L_CC(K, 1) }                                                        \
   break;
   switch (KP) {
-    case 0: L_CT(0)
+    case 0:  // no projections: nothing to test, one tile per CTA
+      if (a.ids) cull_fill_kernel<0><<<(unsigned)T, 256, 0, s>>>(a);
+      else cull_count_kernel<0, 1, true><<<groups, 256, 0, s>>>(a);
+      break;
     case 8: L_CT(8)
     case 16: L_CT(16)
     case 24: L_CT(24)
