@@ -290,8 +290,10 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = tmem_base;
-  const long long beg = s_range[0], end = s_range[1];
-  const int nchunks = (int)((end - beg + NC - 1) / NC);
+  // entries are below 2^31 (the capacity's limit): 32 bits spare registers
+  // (N = 6 fit 24.8 -> 23.2 ms, N = 10 26.2 -> 25.7)
+  const int beg = (int)s_range[0], cnt = (int)(s_range[1] - s_range[0]);
+  const int nchunks = (cnt + NC - 1) / NC;
   const int U = nchunks * nh;
   volatile int* abort_flag = &s_abort;
   auto fail = [&]() {
@@ -308,8 +310,8 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
     for (int d = 0; d < N; ++d) hsc[d] = sh[d];
     // candidate j of chunk i: Gaussian index (or -1) and its entry index (or -1)
     auto cand = [&](int i) -> int2 {
-      const long long e = beg + (long long)i * NC + j;
-      const bool in = i < nchunks && e < end;
+      const int e = beg + i * NC + j;
+      const bool in = i * NC + j < cnt;
       const int g = in ? a.ids[e] : -1;
       const bool live = (unsigned)g < (unsigned)a.Ge;
       const int sl = live ? (int)e : -1;
@@ -463,10 +465,10 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
       // The warp's 32 records are consecutive entries: stage this half of 16
       // records at a time and store with coalesced accesses; entries past the
       // tile's end are not written.
-      const long long w0 = beg + (long long)ic * NC + warp * 32;
-      const long long nval = end - w0 < 32 ? end - w0 : 32;
+      const int r0 = ic * NC + warp * 32;
+      const int nval = cnt - r0 < 32 ? cnt - r0 : 32;
       float4* stg = Outs + warp * (16 * (S::PQMAX + 1));
-      float4* dst = reinterpret_cast<float4*>(a.part) + w0 * S::RQT + p0 / 4;
+      float4* dst = reinterpret_cast<float4*>(a.part) + ((long long)beg + r0) * S::RQT + p0 / 4;
 #pragma unroll
       for (int hb = 0; hb < 2; ++hb) {
         if ((lane >> 4) == hb) {
