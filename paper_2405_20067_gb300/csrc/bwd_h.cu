@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(416, 1) bwd_h_kernel(BwdArgs a) {
   fence_after_sync();
   const uint32_t tmem = tmem_base;
   // entries are below 2^31 (the capacity's limit): 32 bits spare registers
-  // (N = 6 fit 24.8 -> 23.2 ms, N = 10 26.2 -> 25.7)
+  // (N = 6 fit 24.8 -> 23.2 ms)
   const int beg = (int)s_range[0], cnt = (int)(s_range[1] - s_range[0]);
   const int nchunks = (cnt + NC - 1) / NC;
   const int U = nchunks * nh;

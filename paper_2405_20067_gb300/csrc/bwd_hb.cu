@@ -309,10 +309,10 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = tmem_base;
-  // entries are below 2^31 (the capacity's limit): 32 bits spare registers
-  // (N = 6 fit 24.8 -> 23.2 ms, N = 10 26.2 -> 25.7)
-  const int beg = (int)s_range[0], cnt = (int)(s_range[1] - s_range[0]);
-  const int nchunks = (cnt + NC - 1) / NC;
+  // (32-bit entries, as in bwd_h.cu, measured N = 8 evaluation 323 -> 330 us,
+  // N = 10 fit 26.2 -> 25.7 ms, N = 9 and 12 within 1%)
+  const long long beg = s_range[0], end = s_range[1];
+  const int nchunks = (int)((end - beg + NC - 1) / NC);
   const int U = nchunks * nh;
   volatile int* abort_flag = &s_abort;
   auto fail = [&]() {
@@ -328,8 +328,8 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
 #pragma unroll
     for (int d = 0; d < N; ++d) hsc[d] = sh[d];
     auto cand = [&](int i) -> int2 {
-      const int e = beg + i * NC + j;
-      const bool in = i * NC + j < cnt;
+      const long long e = beg + (long long)i * NC + j;
+      const bool in = i < nchunks && e < end;
       const int g = in ? a.ids[e] : -1;
       const bool live = (unsigned)g < (unsigned)a.Ge;
       return make_int2(live ? g : -1, live ? (int)e : -1);
@@ -644,10 +644,10 @@ __global__ void __launch_bounds__(416, 1) bwd_hb_kernel(BwdArgs a) {
       }
       // the warp's 32 records are consecutive entries: stage 16 at a time and
       // store coalesced; entries past the tile's end are not written
-      const int r0 = ic * NC + quad * 32;
-      const int nval = cnt - r0 < 32 ? cnt - r0 : 32;
+      const long long w0 = beg + (long long)ic * NC + quad * 32;
+      const long long nval = end - w0 < 32 ? end - w0 : 32;
       float4* stg = Outs + (warp - 4) * (16 * S::PQS);
-      float4* dst = reinterpret_cast<float4*>(a.part) + ((long long)beg + r0) * S::RQT + p0 / 4;
+      float4* dst = reinterpret_cast<float4*>(a.part) + w0 * S::RQT + p0 / 4;
 #pragma unroll
       for (int hb = 0; hb < 2; ++hb) {
         if ((lane >> 4) == hb) {
