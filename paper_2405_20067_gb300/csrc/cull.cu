@@ -514,10 +514,12 @@ __device__ __forceinline__ long long slice_bound(long long n_src, int w) {
 // Count pass: one CTA per group of TG tiles.  A warp reads 32 key rows once
 // and tests them against every tile of the group, counts the survivors and
 // stores the ballot of every 32 sources in masks[t][i / 32].  Bound by the
-// tests' instructions: up to 128 buckets (SMALL) every byte is below 128, and
+// tests' instructions: up to 128 buckets (SMALL) every bucket is below 128, and
 // with bit 7 set in the minuends a <= b in all four bytes of a word is one
 // subtraction (no byte borrows) whose bits 7 stay; the general byte compares
-// take several instructions each.
+// take several instructions each.  Padding projections hold 0 and 255 on both
+// sides: 255 - 0 passes as well.  Rows of dead Gaussians (255 above 0) would
+// borrow, but lie beyond the last bin and in no run.
 template <int KP, int TG, bool SMALL>
 __global__ void __launch_bounds__(256) cull_count_kernel(CullTileArgs a) {
   constexpr int W = KP / 4;  // 32-bit words per key half (KP >= 8)
